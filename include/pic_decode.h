@@ -87,11 +87,13 @@ typedef enum {
 } pic_latent_format;
 
 typedef enum {
-    /* The library's choice per architecture (measured: TMA where it is as
-     * fast as per-thread copies, per-thread copies where TMA was slower). */
+    /* The library's choice: the row-marching kernels, which load every latent
+     * word of a strip of pixel columns once, one row ahead, by 4-byte
+     * asynchronous copies.  Measured the fastest on every architecture. */
     PIC_STAGING_AUTO = 0,
-    /* Every latent word a tile needs is loaded by the decoding threads'
-     * 4-byte asynchronous copies, one tile ahead. */
+    /* The per-tile kernels: every latent word a tile needs is loaded by the
+     * decoding threads' 4-byte asynchronous copies, one tile ahead.
+     * Architectures that have only a row-marching kernel run that. */
     PIC_STAGING_COPIES = 1,
     /* A tile's full-resolution row (every channel) arrives as TMA boxes
      * issued two tiles ahead; the coarser levels' rows stay with per-thread

@@ -1,6 +1,8 @@
-// k_tc.cuh -- the tensor-core decode kernel template (PIC_PREC_FP16_TC),
-// included by k_tc.cu (int32 latent symbols) and k_tc_f32lat.cu (fp32
-// latents); the two instantiation sets compile in parallel.
+// k_tc.cuh -- the per-tile tensor-core decode kernel template: what a decoder
+// runs that asks for one of its latent stagings (PIC_STAGING_COPIES or _TMA)
+// or for the fp8 lo term (PIC_PREC_FP16_TC_LO8).  PIC_STAGING_AUTO runs the
+// row-marching kernels (k_tcmarch.cuh, k_strip.cuh), which are faster or
+// equal on every net.
 //
 // The synthesis MLP g_s (Sec. 4.1) runs as a chain of tcgen05 MMAs with the
 // accumulators in tensor memory (TMEM); dequantisation, bilinear upsampling

@@ -78,15 +78,30 @@ bool arch_valid(const pic_arch* a) {
   return true;
 }
 
-bool kernel_matches(const KernelInfo& k, const pic_arch* a, bool tma = false) {
-  if (k.generic || (k.tma != 0) != tma || k.precision != a->precision ||
-      k.latent_format != a->latent_format ||
-      k.C != a->channels_per_level ||
-      k.n_layers != a->num_layers || k.act != a->hidden_act)
+bool kernel_matches(const KernelInfo& k, const pic_arch* a) {
+  if (k.generic || k.precision != a->precision || k.latent_format != a->latent_format ||
+      k.C != a->channels_per_level || k.n_layers != a->num_layers || k.act != a->hidden_act)
     return false;
   for (int i = 0; i <= a->num_layers; ++i)
     if (k.dims[i] != a->dims[i]) return false;
   return true;
+}
+
+// The arch's specialised kernel among table[0, n): without `tma` its
+// row-marching kernel -- it is the faster one for every net that has both --
+// or, where the caller asked for a staging of the per-tile kernels
+// (PIC_STAGING_COPIES or _TMA), the per-tile one if there is one; with `tma`
+// the per-tile kernel's TMA-staged twin, only where the caller asked for it.
+const KernelInfo* find_kernel(const KernelInfo* table, int n, const pic_arch* a, bool tma) {
+  if (tma && a->staging != PIC_STAGING_TMA) return nullptr;
+  const bool want_march = !tma && a->staging == PIC_STAGING_AUTO;
+  const KernelInfo* other = nullptr;
+  for (int i = 0; i < n && i < 32; ++i) {
+    if (!kernel_matches(table[i], a) || (table[i].tma != 0) != tma) continue;
+    if ((table[i].march != 0) == want_march) return &table[i];
+    if (!other) other = &table[i];
+  }
+  return other;
 }
 
 bool aligned(const void* p, uintptr_t a) { return (reinterpret_cast<uintptr_t>(p) % a) == 0; }
@@ -297,12 +312,7 @@ int pic_decode_create(const pic_arch* arch, pic_decoder** out) {
   // else (fp32 only) the generic kernel.
   KernelInfo table[32];
   int n = arch->precision == PIC_PREC_FP32 ? pic::fp32_kernels(table, 32) : pic::tc_kernels(table, 32);
-  const KernelInfo* chosen = nullptr;
-  for (int i = 0; i < n && i < 32; ++i)
-    if (kernel_matches(table[i], arch)) {
-      chosen = &table[i];
-      break;
-    }
+  const KernelInfo* chosen = find_kernel(table, n, arch, false);
   KernelInfo k{};
   if (chosen) {
     k = *chosen;
@@ -327,16 +337,9 @@ int pic_decode_create(const pic_arch* arch, pic_decoder** out) {
     return PIC_ERR_UNSUPPORTED;
   }
 
-  // the TMA-staged twin, where the arch has one
-  const KernelInfo* twin = nullptr;
+  // the TMA-staged twin, where it is asked for
+  const KernelInfo* twin = find_kernel(table, n, arch, true);
   int per_sm_tma = 0;
-  for (int i = 0; i < n && i < 32; ++i)
-    if (kernel_matches(table[i], arch, true)) {
-      twin = &table[i];
-      break;
-    }
-  if (arch->staging == PIC_STAGING_COPIES || (arch->staging == PIC_STAGING_AUTO && twin && !twin->tma_default))
-    twin = nullptr;
   if (arch->staging == PIC_STAGING_TMA && !twin) return PIC_ERR_UNSUPPORTED;
   if (twin && (twin->smem_bytes > static_cast<int>(prop.sharedMemPerBlockOptin) || !regs_match(*twin) ||
                cudaFuncSetAttribute(twin->fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -345,8 +348,7 @@ int pic_decode_create(const pic_arch* arch, pic_decoder** out) {
                                                              twin->smem_bytes) != cudaSuccess ||
                per_sm_tma < 1)) {
     cudaGetLastError();
-    if (arch->staging == PIC_STAGING_TMA) return PIC_ERR_UNSUPPORTED;
-    twin = nullptr;  // the per-thread-copy kernel serves every call
+    return PIC_ERR_UNSUPPORTED;
   }
 
   pic_decoder* h = new (std::nothrow) pic_decoder();
@@ -717,12 +719,7 @@ extern "C" int pic_decode_batch_noalloc(const pic_arch* arch, int B, const int32
   // on this stack frame.
   KernelInfo table[32];
   int n = arch->precision == PIC_PREC_FP32 ? pic::fp32_kernels(table, 32) : pic::tc_kernels(table, 32);
-  const KernelInfo* chosen = nullptr;
-  for (int i = 0; i < n && i < 32; ++i)
-    if (kernel_matches(table[i], arch)) {
-      chosen = &table[i];
-      break;
-    }
+  const KernelInfo* chosen = find_kernel(table, n, arch, false);
   pic_decoder h{};
   h.arch = *arch;
   h.device = dev;
@@ -744,19 +741,14 @@ extern "C" int pic_decode_batch_noalloc(const pic_arch* arch, int B, const int32
   h.grid_cap = per_sm * d.sms;
   // the TMA-staged twin, as pic_decode_create picks it (its tensor maps are
   // encoded on the host for each call: no device memory)
-  for (int i = 0; i < n && i < 32; ++i)
-    if (kernel_matches(table[i], arch, true)) {
-      if (arch->staging == PIC_STAGING_COPIES ||
-          (arch->staging == PIC_STAGING_AUTO && !table[i].tma_default))
-        break;
-      int per_sm_tma = 0;
-      if (table[i].smem_bytes <= d.smem_optin && noalloc_kernel(dev, table[i], &per_sm_tma) == PIC_OK) {
-        h.has_tma = true;
-        h.kern_tma = table[i];
-        h.grid_cap_tma = per_sm_tma * d.sms;
-      }
-      break;
+  if (const KernelInfo* twin = find_kernel(table, n, arch, true)) {
+    int per_sm_tma = 0;
+    if (twin->smem_bytes <= d.smem_optin && noalloc_kernel(dev, *twin, &per_sm_tma) == PIC_OK) {
+      h.has_tma = true;
+      h.kern_tma = *twin;
+      h.grid_cap_tma = per_sm_tma * d.sms;
     }
+  }
   if (arch->staging == PIC_STAGING_TMA && !h.has_tma) return PIC_ERR_UNSUPPORTED;
   h.n_params = pic_param_count(arch);
   h.d_status = d.scratch;

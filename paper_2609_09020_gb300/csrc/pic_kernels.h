@@ -19,7 +19,7 @@ struct KernelInfo {
   int smem_bytes;  // dynamic shared memory per CTA
   int tile_px;     // pixels per tile (one tile = a run of one image row)
   int tma;         // 1: stages the latents with TMA (needs valid TmaParams)
-  int tma_default; // (TMA kernels) 1: PIC_STAGING_AUTO picks it over its per-thread-copy twin
+  int march;       // 1: a row-marching kernel (what PIC_STAGING_AUTO runs where there is one)
   const void* fn;  // __global__ function taking (DecodeParams), or (DecodeParams,
                    // TmaParams) for the tensor-core kernels (precision 1)
 };
@@ -27,9 +27,10 @@ struct KernelInfo {
 int fp32_kernels(KernelInfo* out, int cap);        // all of them
 int fp32_kernels_sweep(KernelInfo* out, int cap);  // the width ablation's (own translation unit)
 KernelInfo fp32_generic_kernel_info(int latent_format);
-int tc_kernels(KernelInfo* out, int cap);     // both latent formats
-int tc_kernels_fp32lat(KernelInfo* out, int cap);  // the fp32-latent ones (own translation unit)
-int tc_kernels_sweep(KernelInfo* out, int cap);    // the width ablation's (own translation unit)
+int tc_kernels(KernelInfo* out, int cap);     // all tensor-core kernels
+int march_kernels(KernelInfo* out, int cap);         // row-marching, 64-wide nets
+int march_kernels_f32lat(KernelInfo* out, int cap);  // the same for fp32 latents
+int strip_kernels(KernelInfo* out, int cap);         // row-marching, narrow nets
 int tc_kernels_tma(KernelInfo* out, int cap);      // TMA-staged variants (own translation unit)
 
 }  // namespace pic
