@@ -23,7 +23,17 @@ int fp32_kernels(KernelInfo* out, int cap) {
   return k;
 }
 
-KernelInfo fp32_generic_kernel_info(int latent_format) {
+namespace {
+template <bool FL>
+const void* any_fn(int t2) {
+  if (t2 <= 2) return reinterpret_cast<const void*>(&fp32_any_kernel<2, FL>);
+  if (t2 <= 5) return reinterpret_cast<const void*>(&fp32_any_kernel<5, FL>);
+  if (t2 <= 8) return reinterpret_cast<const void*>(&fp32_any_kernel<8, FL>);
+  return reinterpret_cast<const void*>(&fp32_any_kernel<16, FL>);
+}
+}  // namespace
+
+KernelInfo fp32_generic_kernel_info(int latent_format, int n_layers, const int* dims, long long params, int max_smem) {
   KernelInfo k{};
   k.name = latent_format ? "fp32_generic_f32lat" : "fp32_generic";
   k.precision = 0;
@@ -31,9 +41,17 @@ KernelInfo fp32_generic_kernel_info(int latent_format) {
   k.generic = 1;
   k.threads = kThreads;
   k.tile_px = kThreads;
-  k.smem_bytes = 0;  // set per arch: params_per_image * 4
-  k.fn = latent_format ? reinterpret_cast<const void*>(&fp32_generic_kernel<true>)
-                      : reinterpret_cast<const void*>(&fp32_generic_kernel<false>);
+  int t2 = 1;
+  const long long tiled = 4 * any_smem_floats(n_layers, dims, &t2);
+  if (tiled <= max_smem) {
+    k.smem_bytes = static_cast<int>(tiled);
+    k.fn = latent_format ? any_fn<true>(t2) : any_fn<false>(t2);
+  } else {
+    k.smem_bytes = params * 4 <= max_smem ? static_cast<int>(params * 4) : max_smem + 1;  // refused by the caller
+    k.fn = latent_format ? reinterpret_cast<const void*>(&fp32_flat_kernel<true>)
+                        : reinterpret_cast<const void*>(&fp32_flat_kernel<false>);
+  }
+  k.smem_attr = max_smem;  // one function serves nets of many sizes
   return k;
 }
 

@@ -197,6 +197,30 @@ __device__ __forceinline__ void store_out_partials(float* __restrict__ X, const 
         make_float4(part[c][0], part[c][1], part[c][2], part[c][3]);
 }
 
+// The tiles of a CTA's contiguous range (fewer than 2^31: each writes at least
+// a pixel), image-major, row-major within an image: two divisions at the
+// range's start, then a cursor.  Two 64-bit divisions per tile and thread,
+// instead, measured 8 % on 14-64-64-3 at 1920x1080 (432 against 398 us), 2 %
+// on 16-64-64-64-3 and 8-32-32-32-3; 7-64-64-3 takes the same time.
+struct TileCursor {
+  int b, y, tx;
+  __device__ __forceinline__ TileCursor(const DecodeParams& p, long long t) {
+    b = static_cast<int>(t / p.tiles_per_image);
+    const long long r = t - static_cast<long long>(b) * p.tiles_per_image;
+    y = static_cast<int>(r / p.tiles_per_row);
+    tx = static_cast<int>(r - static_cast<long long>(y) * p.tiles_per_row);
+  }
+  __device__ __forceinline__ void next(const DecodeParams& p) {
+    if (++tx == p.tiles_per_row) {
+      tx = 0;
+      if (++y == p.H) {
+        y = 0;
+        ++b;
+      }
+    }
+  }
+};
+
 template <int C, int NL, int D0, int D1, int D2, int D3, int D4, int ACT>
 struct Fp32Net {
   static_assert(NL >= 2 && NL <= 4, "1 to 3 hidden layers");
@@ -427,8 +451,7 @@ __global__ void __launch_bounds__(kThreads) fp32_px_kernel(const DecodeParams p)
     const int b = static_cast<int>(t / p.tiles_per_image);
     const long long r = t - static_cast<long long>(b) * p.tiles_per_image;
     const int y = static_cast<int>(r / p.tiles_per_row);
-    const int x = static_cast<int>(r - static_cast<long long>(y) * p.tiles_per_row) * kThreads +
-                  threadIdx.x;
+    const int x = static_cast<int>(r - static_cast<long long>(y) * p.tiles_per_row) * kThreads + threadIdx.x;
     if (b != cur_b) {  // uniform across the CTA
       __syncthreads();
       const float* w = wts + b * p.params_per_image;
@@ -488,11 +511,226 @@ __global__ void __launch_bounds__(kThreads) fp32_px_kernel(const DecodeParams p)
 }
 
 // ---------------------------------------------------------------------------
-// Generic kernel: any dims up to kMaxDim, runtime loops, weights in shared
-// memory in the nn.Linear layout.  Slower (hidden values in local memory) but
-// covers every arch the C ABI accepts.
+// Any net (runtime dims): the register-tiled contraction above with the
+// widths read at run time.  Warp ng of the CTA owns a quarter of a layer's
+// neurons, rounded up to a pair count tn2 that picks one of the unrolled
+// inner loops (any_layer), and its lane 4 pixels; padding neurons have zero
+// weights.  The output layer is one thread per pixel.  Every sum runs over
+// the inputs in order from the bias, one FMA each, as in fp32_flat_kernel.
+//
+// It replaced one thread per pixel with the hidden values in local memory
+// (fp32_flat_kernel below), which made two local-memory and one shared-memory
+// access per FMA; 4 images of 768x512: 5-24-24-3 376 -> 101 us, 6-8-8-3
+// 118 -> 58 us; two 512x512 GELU images of 6-37-30-12-3 299 -> 89 us.  The
+// contraction is 60 % of the rest (about 880 instructions per 128 pixels and
+// warp for 5-24-24-3, a third of them the FMAs), the features 15 %.  Measured
+// and dropped: weights twice in shared memory and FMA pairs over pixels
+// instead of the operands' duplicating moves (115 us), marching down the rows
+// with the interpolated source rows in shared memory (115 us with it).
+// MAXT2 bounds tn2 (widths up to 8 MAXT2), so that narrow nets are not held
+// to the wide ones' registers.
+
+__host__ __device__ constexpr int any_segf(int tn2) { return (2 * tn2 + 3) / 4 * 4; }  // floats per warp and row
+__host__ __device__ constexpr int any_tn2(int width) {  // pairs per warp, an unrolled count
+  return (width + 7) / 8 <= 8 ? (width + 7) / 8 : ((width + 7) / 8 + 3) / 4 * 4;
+}
+// Shared memory of a net: per hidden layer K weight rows and the bias row of
+// 4 segments; the output layer's K + 1 rows of 4; X.
+inline long long any_smem_floats(int n_layers, const int* dims, int* max_t2) {
+  long long w = 0;
+  int rows = dims[0], m = 1;
+  for (int k = 0; k + 1 < n_layers; ++k) {
+    const int t2 = any_tn2(dims[k + 1]);
+    w += (dims[k] + 1LL) * kWarps * any_segf(t2);
+    if (8 * t2 > rows) rows = 8 * t2;
+    if (t2 > m) m = t2;
+  }
+  *max_t2 = m;
+  return w + (dims[n_layers - 1] + 1LL) * 4 + static_cast<long long>(rows) * kThreads;
+}
+
+// One hidden layer of K inputs: X rows [0, K) -> X rows [0, 8 TN2).
+template <int TN2>
+__device__ __forceinline__ void any_layer(float* __restrict__ X, const float* __restrict__ wl, int K, int lane,
+                                          int warp, int act) {
+  constexpr int SEGF = any_segf(TN2), NCH = SEGF / 4, ROWF = kWarps * SEGF;
+  const float* w = wl + warp * SEGF;
+  unsigned long long acc[kTP][TN2];
+  {
+    const float* bias = w + K * ROWF;
+#pragma unroll
+    for (int j = 0; j < TN2; ++j) {
+      const unsigned long long v = *reinterpret_cast<const unsigned long long*>(bias + 2 * j);
+#pragma unroll
+      for (int p = 0; p < kTP; ++p) acc[p][j] = v;
+    }
+  }
+  const float* xa = X + 4 * lane;
+#pragma unroll 4
+  for (int k = 0; k < K; ++k) {
+    const float4 a = *reinterpret_cast<const float4*>(xa + k * kThreads);
+    unsigned long long wv[2 * NCH];
+#pragma unroll
+    for (int c = 0; c < NCH; ++c) {
+      const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(w + k * ROWF + 4 * c);
+      wv[2 * c] = v.x;
+      wv[2 * c + 1] = v.y;
+    }
+    const unsigned long long ad[kTP] = {pack2(a.x, a.x), pack2(a.y, a.y), pack2(a.z, a.z), pack2(a.w, a.w)};
+#pragma unroll
+    for (int p = 0; p < kTP; ++p)
+#pragma unroll
+      for (int j = 0; j < TN2; ++j) acc[p][j] = fma2(wv[j], ad[p], acc[p][j]);
+  }
+  if (act == ACT_GELU) {
+#pragma unroll
+    for (int p = 0; p < kTP; ++p)
+#pragma unroll
+      for (int j = 0; j < TN2; ++j) acc[p][j] = gelu_approx2(acc[p][j]);
+  } else {
+#pragma unroll
+    for (int p = 0; p < kTP; ++p)
+#pragma unroll
+      for (int j = 0; j < TN2; ++j) {
+        const float2 v = unpack2(acc[p][j]);
+        acc[p][j] = pack2(fmaxf(v.x, 0.0f), fmaxf(v.y, 0.0f));
+      }
+  }
+  __syncthreads();  // every warp has read X
+#pragma unroll
+  for (int j = 0; j < 2 * TN2; ++j)
+    *reinterpret_cast<float4*>(X + (warp * 2 * TN2 + j) * kThreads + 4 * lane) =
+        make_float4(half_of(acc[0][j >> 1], j & 1), half_of(acc[1][j >> 1], j & 1), half_of(acc[2][j >> 1], j & 1),
+                    half_of(acc[3][j >> 1], j & 1));
+  __syncthreads();
+}
+
+constexpr int kAnyBatch = 4;
+
+template <int MAXT2, bool FL>
+__global__ void __launch_bounds__(kThreads, MAXT2 <= 5 ? 5 : (MAXT2 <= 8 ? 4 : 2))
+    fp32_any_kernel(const DecodeParams p) {
+  extern __shared__ __align__(16) float smem[];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  int w_floats = (p.dims[p.n_layers - 1] + 1) * 4;
+  for (int k = 0; k + 1 < p.n_layers; ++k) w_floats += (p.dims[k] + 1) * kWarps * any_segf(any_tn2(p.dims[k + 1]));
+  float* const X = smem + w_floats;
+  const long long t_begin = blockIdx.x * p.total_tiles / gridDim.x;
+  const long long t_end = (blockIdx.x + 1LL) * p.total_tiles / gridDim.x;
+  const float* wts = static_cast<const float*>(p.weights);
+  int cur_b = -1;
+  TileCursor cur(p, t_begin);
+  for (int left = static_cast<int>(t_end - t_begin); left > 0; --left) {
+    const int b = cur.b, y = cur.y;
+    const int x = cur.tx * kThreads + tid;
+    cur.next(p);
+    if (b != cur_b) {
+      __syncthreads();
+      const float* w = wts + b * p.params_per_image;
+      float* sm = smem;
+      for (int l = 0; l + 1 < p.n_layers; ++l) {
+        const int K = p.dims[l], N = p.dims[l + 1], tn2 = any_tn2(N), segf = any_segf(tn2), rowf = kWarps * segf;
+        for (int e = tid; e < (K + 1) * rowf; e += kThreads) {
+          const int k = e / rowf, q = e - k * rowf, ng = q / segf, j = q - ng * segf;
+          const int n = ng * 2 * tn2 + j;
+          sm[e] = j < 2 * tn2 && n < N ? (k < K ? __ldg(w + n * K + k) : __ldg(w + N * K + n)) : 0.0f;
+        }
+        sm += (K + 1) * rowf;
+        w += N * K + N;
+      }
+      const int K = p.dims[p.n_layers - 1];
+      for (int e = tid; e < (K + 1) * 4; e += kThreads) {
+        const int k = e >> 2, c = e & 3;
+        sm[e] = c < 3 ? (k < K ? __ldg(w + c * K + k) : __ldg(w + 3 * K + c)) : 0.0f;
+      }
+      cur_b = b;
+      __syncthreads();
+    }
+    {
+      const int xc = min(x, p.W - 1);  // pixels past the row's end decode column W - 1 and are not stored
+      const int32_t* lat = p.latents + b * p.lat_per_image;
+      // level 0 has the output size: the upsampling is the identity
+      const float s0 = FL ? 1.0f : __ldg(p.steps + b * p.L);
+      const long long plane = static_cast<long long>(p.H) * p.W;
+      for (int c = 0; c < p.C; ++c)
+        X[c * kThreads + tid] = s0 * lat_value<FL>(__ldg(lat + c * plane + static_cast<long long>(y) * p.W + xc));
+      // the others kAnyBatch features at a time, all their loads in flight together
+      const int D0 = p.L * p.C;
+      int l = 1, c = 0;
+      for (int i = p.C; i < D0; i += kAnyBatch) {
+        int q[kAnyBatch][4];
+        float fx[kAnyBatch], fy[kAnyBatch], st[kAnyBatch];
+#pragma unroll
+        for (int u = 0; u < kAnyBatch; ++u) {
+          if (i + u < D0) {
+            const LevelGeom& lg = p.lv[l];
+            const Tap tx = bilinear_tap(xc, lg.sx, lg.W);
+            const Tap ty = bilinear_tap(y, lg.sy, lg.H);
+            const int32_t* pl = lat + lg.off + static_cast<long long>(c) * lg.H * lg.W;
+            const int32_t* r0 = pl + static_cast<long long>(ty.i0) * lg.W;
+            const int32_t* r1 = pl + static_cast<long long>(ty.i1) * lg.W;
+            q[u][0] = __ldg(r0 + tx.i0);
+            q[u][1] = __ldg(r0 + tx.i1);
+            q[u][2] = __ldg(r1 + tx.i0);
+            q[u][3] = __ldg(r1 + tx.i1);
+            fx[u] = tx.frac;
+            fy[u] = ty.frac;
+            st[u] = FL ? 1.0f : __ldg(p.steps + b * p.L + l);
+            if (++c == p.C) {
+              c = 0;
+              ++l;
+            }
+          }
+        }
+#pragma unroll
+        for (int u = 0; u < kAnyBatch; ++u)
+          if (i + u < D0) {
+            const float top = lat_lerp<FL>(q[u][0], q[u][1], fx[u]), bot = lat_lerp<FL>(q[u][2], q[u][3], fx[u]);
+            X[(i + u) * kThreads + tid] = st[u] * fmaf(fy[u], bot - top, top);
+          }
+      }
+    }
+    __syncthreads();
+    const float* wl = smem;
+    for (int l = 0; l + 1 < p.n_layers; ++l) {
+      const int K = p.dims[l], tn2 = any_tn2(p.dims[l + 1]);
+      switch (tn2) {
+        case 1: any_layer<1>(X, wl, K, lane, warp, p.act); break;
+        case 2: any_layer<2>(X, wl, K, lane, warp, p.act); break;
+        case 3: if constexpr (MAXT2 >= 3) any_layer<3>(X, wl, K, lane, warp, p.act); break;
+        case 4: if constexpr (MAXT2 >= 4) any_layer<4>(X, wl, K, lane, warp, p.act); break;
+        case 5: if constexpr (MAXT2 >= 5) any_layer<5>(X, wl, K, lane, warp, p.act); break;
+        case 6: if constexpr (MAXT2 >= 6) any_layer<6>(X, wl, K, lane, warp, p.act); break;
+        case 7: if constexpr (MAXT2 >= 7) any_layer<7>(X, wl, K, lane, warp, p.act); break;
+        case 8: if constexpr (MAXT2 >= 8) any_layer<8>(X, wl, K, lane, warp, p.act); break;
+        case 12: if constexpr (MAXT2 >= 12) any_layer<12>(X, wl, K, lane, warp, p.act); break;
+        default: if constexpr (MAXT2 >= 16) any_layer<16>(X, wl, K, lane, warp, p.act); break;
+      }
+      wl += (K + 1) * kWarps * any_segf(tn2);
+    }
+    {  // output layer of pixel tid
+      const int K = p.dims[p.n_layers - 1];
+      const float4 bo = *reinterpret_cast<const float4*>(wl + 4 * K);
+      float o0 = bo.x, o1 = bo.y, o2 = bo.z;
+#pragma unroll 4
+      for (int k = 0; k < K; ++k) {
+        const float4 wv = *reinterpret_cast<const float4*>(wl + 4 * k);
+        const float h = X[k * kThreads + tid];
+        o0 = fmaf(wv.x, h, o0);
+        o1 = fmaf(wv.y, h, o1);
+        o2 = fmaf(wv.z, h, o2);
+      }
+      if (x < p.W) store_rgb(p, b, y, x, o0, o1, o2);
+    }
+    __syncthreads();  // X is free for the next tile
+  }
+}
+
+// Nets whose padded weights and activation buffer exceed the shared memory
+// (widths beyond 100 in several layers): weights in shared memory in the
+// nn.Linear layout, one thread per pixel, hidden values in local memory.
 template <bool FL>
-__global__ void __launch_bounds__(kThreads) fp32_generic_kernel(const DecodeParams p) {
+__global__ void __launch_bounds__(kThreads) fp32_flat_kernel(const DecodeParams p) {
   extern __shared__ __align__(16) float sm_w[];
   // balanced contiguous ranges: every CTA gets floor or ceil of tiles / CTAs
   const long long t_begin = blockIdx.x * p.total_tiles / gridDim.x;
@@ -503,8 +741,7 @@ __global__ void __launch_bounds__(kThreads) fp32_generic_kernel(const DecodePara
     const int b = static_cast<int>(t / p.tiles_per_image);
     const long long r = t - static_cast<long long>(b) * p.tiles_per_image;
     const int y = static_cast<int>(r / p.tiles_per_row);
-    const int x = static_cast<int>(r - static_cast<long long>(y) * p.tiles_per_row) * kThreads +
-                  threadIdx.x;
+    const int x = static_cast<int>(r - static_cast<long long>(y) * p.tiles_per_row) * kThreads + threadIdx.x;
     if (b != cur_b) {
       __syncthreads();
       for (long long e = threadIdx.x; e < p.params_per_image; e += blockDim.x)

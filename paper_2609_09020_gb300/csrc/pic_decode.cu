@@ -317,15 +317,15 @@ int pic_decode_create(const pic_arch* arch, pic_decoder** out) {
   if (chosen) {
     k = *chosen;
   } else if (arch->precision == PIC_PREC_FP32) {
-    k = pic::fp32_generic_kernel_info(arch->latent_format);
-    k.smem_bytes = static_cast<int>(pic_param_count(arch) * 4);
+    k = pic::fp32_generic_kernel_info(arch->latent_format, arch->num_layers, arch->dims, pic_param_count(arch),
+                                      static_cast<int>(prop.sharedMemPerBlockOptin));
   } else {
     return PIC_ERR_UNSUPPORTED;
   }
   if (k.smem_bytes > static_cast<int>(prop.sharedMemPerBlockOptin)) return PIC_ERR_UNSUPPORTED;
   if (!regs_match(k)) return PIC_ERR_UNSUPPORTED;
-  if (cudaFuncSetAttribute(k.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, k.smem_bytes) !=
-      cudaSuccess) {
+  if (cudaFuncSetAttribute(k.fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           k.smem_attr ? k.smem_attr : k.smem_bytes) != cudaSuccess) {
     cudaGetLastError();
     return PIC_ERR_CUDA;
   }
@@ -619,6 +619,7 @@ struct NoallocDevice {
 struct NoallocKernel {
   int dev;
   const void* fn;
+  int smem;  // (a generic kernel serves nets of several sizes)
   int per_sm;
   bool regs_ok;
 };
@@ -664,15 +665,15 @@ int noalloc_device(int dev, NoallocDevice* out) {
 int noalloc_kernel(int dev, const KernelInfo& k, int* per_sm) {
   std::lock_guard<std::mutex> lock(g_noalloc_mutex);
   for (int i = 0; i < g_noalloc_nkern; ++i)
-    if (g_noalloc_kern[i].dev == dev && g_noalloc_kern[i].fn == k.fn) {
+    if (g_noalloc_kern[i].dev == dev && g_noalloc_kern[i].fn == k.fn && g_noalloc_kern[i].smem == k.smem_bytes) {
       if (!g_noalloc_kern[i].regs_ok) return PIC_ERR_UNSUPPORTED;
       *per_sm = g_noalloc_kern[i].per_sm;
       return PIC_OK;
     }
-  NoallocKernel e{dev, k.fn, 0, regs_match(k)};
+  NoallocKernel e{dev, k.fn, k.smem_bytes, 0, regs_match(k)};
   if (e.regs_ok) {
-    if (cudaFuncSetAttribute(k.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, k.smem_bytes) !=
-        cudaSuccess) {
+    if (cudaFuncSetAttribute(k.fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             k.smem_attr ? k.smem_attr : k.smem_bytes) != cudaSuccess) {
       cudaGetLastError();
       return PIC_ERR_CUDA;
     }
@@ -727,8 +728,8 @@ extern "C" int pic_decode_batch_noalloc(const pic_arch* arch, int B, const int32
   if (chosen) {
     h.kern = *chosen;
   } else if (arch->precision == PIC_PREC_FP32) {
-    h.kern = pic::fp32_generic_kernel_info(arch->latent_format);
-    h.kern.smem_bytes = static_cast<int>(pic_param_count(arch) * 4);
+    h.kern = pic::fp32_generic_kernel_info(arch->latent_format, arch->num_layers, arch->dims,
+                                           pic_param_count(arch), d.smem_optin);
   } else {
     return PIC_ERR_UNSUPPORTED;
   }

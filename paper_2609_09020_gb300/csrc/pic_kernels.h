@@ -17,6 +17,7 @@ struct KernelInfo {
   int threads;     // threads per CTA
   int regs_at_launch;  // registers per thread the kernel must be built with (0: any)
   int smem_bytes;  // dynamic shared memory per CTA
+  int smem_attr;   // the function's shared-memory attribute, where it serves several sizes (0: smem_bytes)
   int tile_px;     // pixels per tile (one tile = a run of one image row)
   int tma;         // 1: stages the latents with TMA (needs valid TmaParams)
   int march;       // 1: a row-marching kernel (what PIC_STAGING_AUTO runs where there is one)
@@ -26,7 +27,9 @@ struct KernelInfo {
 
 int fp32_kernels(KernelInfo* out, int cap);        // all of them
 int fp32_kernels_sweep(KernelInfo* out, int cap);  // the width ablation's (own translation unit)
-KernelInfo fp32_generic_kernel_info(int latent_format);
+// the kernel for an fp32 net without one of its own; its smem_bytes exceeds
+// max_smem (the device's limit per block) if the net does not fit any
+KernelInfo fp32_generic_kernel_info(int latent_format, int n_layers, const int* dims, long long params, int max_smem);
 int tc_kernels(KernelInfo* out, int cap);     // all tensor-core kernels
 int march_kernels(KernelInfo* out, int cap);         // row-marching, 64-wide nets
 int march_kernels_f32lat(KernelInfo* out, int cap);  // the same for fp32 latents
