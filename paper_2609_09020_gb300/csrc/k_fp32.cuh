@@ -268,11 +268,11 @@ __global__ void __launch_bounds__(kThreads, (Fp32Net<C, NL, D0, D1, D2, D3, D4, 
   const long long plane = static_cast<long long>(p.H) * p.W;
   int cur_b = -1;
 
-  for (long long t = t_begin; t < t_end; ++t) {
-    const int b = static_cast<int>(t / p.tiles_per_image);
-    const long long r = t - static_cast<long long>(b) * p.tiles_per_image;
-    const int y = static_cast<int>(r / p.tiles_per_row);
-    const int x = static_cast<int>(r - static_cast<long long>(y) * p.tiles_per_row) * kThreads + tid;
+  TileCursor cur(p, t_begin);
+  for (int left = static_cast<int>(t_end - t_begin); left > 0; --left) {
+    const int b = cur.b, y = cur.y;
+    const int x = cur.tx * kThreads + tid;
+    cur.next(p);
     if (b != cur_b) {  // uniform across the CTA
       __syncthreads();
       const float* w = wts + b * p.params_per_image;
@@ -447,11 +447,11 @@ __global__ void __launch_bounds__(kThreads) fp32_px_kernel(const DecodeParams p)
   const long long plane = static_cast<long long>(p.H) * p.W;
   int cur_b = -1;
 
-  for (long long t = t_begin; t < t_end; ++t) {
-    const int b = static_cast<int>(t / p.tiles_per_image);
-    const long long r = t - static_cast<long long>(b) * p.tiles_per_image;
-    const int y = static_cast<int>(r / p.tiles_per_row);
-    const int x = static_cast<int>(r - static_cast<long long>(y) * p.tiles_per_row) * kThreads + threadIdx.x;
+  TileCursor cur(p, t_begin);
+  for (int left = static_cast<int>(t_end - t_begin); left > 0; --left) {
+    const int b = cur.b, y = cur.y;
+    const int x = cur.tx * kThreads + threadIdx.x;
+    cur.next(p);
     if (b != cur_b) {  // uniform across the CTA
       __syncthreads();
       const float* w = wts + b * p.params_per_image;
@@ -737,11 +737,11 @@ __global__ void __launch_bounds__(kThreads) fp32_flat_kernel(const DecodeParams 
   const long long t_end = (blockIdx.x + 1LL) * p.total_tiles / gridDim.x;
   const float* wts = static_cast<const float*>(p.weights);
   int cur_b = -1;
-  for (long long t = t_begin; t < t_end; ++t) {
-    const int b = static_cast<int>(t / p.tiles_per_image);
-    const long long r = t - static_cast<long long>(b) * p.tiles_per_image;
-    const int y = static_cast<int>(r / p.tiles_per_row);
-    const int x = static_cast<int>(r - static_cast<long long>(y) * p.tiles_per_row) * kThreads + threadIdx.x;
+  TileCursor cur(p, t_begin);
+  for (int left = static_cast<int>(t_end - t_begin); left > 0; --left) {
+    const int b = cur.b, y = cur.y;
+    const int x = cur.tx * kThreads + threadIdx.x;
+    cur.next(p);
     if (b != cur_b) {
       __syncthreads();
       for (long long e = threadIdx.x; e < p.params_per_image; e += blockDim.x)
