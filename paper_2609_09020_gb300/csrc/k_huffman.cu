@@ -2,36 +2,55 @@
 // (include/pic_huffman.h; Sec. 3.3 and Sec. 4.1 of the paper, which adapts
 // GPUHD, Weissenberger & Schmidt 2018: self-synchronising parallel decoding).
 //
-// 1. huff_lut (one CTA per image): the stored table -- values and lengths in
-//    canonical order -- is the run-length code of the 2^p-entry lookup table:
-//    symbol k covers 2^(p - len_k) consecutive entries.  Expanding the runs
-//    gives the table (16-bit entry = length << 12 | k, the symbol's row in
-//    the stored table, whose value is read only when it is written out), so
-//    one lookup of the next p bits decodes a symbol.  Kraft's inequality is
-//    checked here.
-// 2. huff_decode (one cooperative launch; every CTA resident, grid-wide
-//    barriers between the phases):
+// One cooperative launch (every CTA resident, grid-wide barriers between the
+// phases):
+//    0. tables: the CTAs expand the stored tables, up to kMaxParts CTAs to an
+//       image.  A table -- values and lengths in canonical order -- is the
+//       run-length code of the 2^p-entry lookup table: symbol k covers
+//       2^(p - len_k) consecutive entries.  Expanding the runs gives the table,
+//       so one lookup of the next p bits decodes a symbol.  A 16-bit entry is
+//       value << 4 | length; where a value takes more than 12 bits the image's
+//       entries are row << 4 | length, the row in the stored table, whose value
+//       is then read when it is written out.  Kraft's inequality is checked
+//       here.  A second table holds, for every p-bit window, how many codewords
+//       lie wholly inside it and the bits they take (one byte: 2.4 codewords on
+//       average where one takes 4.3 bits), which is all that counting needs.
 //    a. each thread decodes its 256-bit subsequences speculatively from their
 //       first bit, which may lie inside a codeword, until it passes the
-//       subsequence's end; it records the first codeword boundary at or
-//       after the end (the exit) and the number of codewords started;
-//    b. synchronisation passes: a subsequence whose start differs from its
-//       predecessor's exit is decoded again from that exit.  Prefix codes
-//       resynchronise within a few codewords, so the passes stop changing
-//       after one or two; pass i has made subsequence i exact, and after 64
-//       passes without convergence the status word says so;
-//    c. an exclusive scan of the codeword counts gives every subsequence's
-//       output position (each image's must equal its symbol offset);
-//    d. every subsequence is decoded from its final start, writing values.
-// Each CTA stages its images' lookup tables and, per pass, the stream words
-// of its 256 subsequences in shared memory.  Each thread keeps a 64-bit
-// window of the stream in registers and reloads one word when its position
-// crosses a word boundary (codes are at most 12 bits, so at most one word per
-// codeword).  The counting decodes of a and b use a pair table per image (the
-// lengths of the first two codewords of every p-bit window, when both lie
-// inside it), so one lookup advances over up to two codewords.  The final
-// decode d writes through per-warp staging rows, 16 symbols per thread per
-// round, so that each warp store writes two whole 64-byte runs.
+//       subsequence's end; it records how far past the end the first
+//       codeword boundary lies (the overshoot, below 12 bits);
+//    b. synchronisation passes: a subsequence whose predecessor's overshoot
+//       differs from the one it was decoded with is decoded again from there
+//       (in the first pass every one is, and counts its codewords).
+//       Prefix codes resynchronise within a few codewords, so a pass seldom
+//       changes an overshoot, and the passes end with the first that changes
+//       none (usually the first); pass i has made subsequence i exact, and
+//       after 64 passes without convergence the status word says so.  Each
+//       pass also leaves the CTAs' codeword totals, from which
+//    c. every CTA takes its output position (the total must equal the symbol
+//       offsets');
+//    d. every subsequence is decoded from its final start, writing values
+//       through per-warp staging rows, so that a warp store writes a run of
+//       one subsequence's values instead of 32 scattered words.
+// Each CTA holds its images' tables in shared memory; each warp goes through
+// groups of 32 subsequences of its own, whose stream words it stages in
+// shared memory (9 words apart: equal words of neighbouring subsequences fall
+// into different banks, and the ninth is the word that follows) without a CTA
+// barrier.
+//
+// What bounds it: for one image latency -- 3 grid barriers, the tables, and a
+// subsequence's serial chain (window, lookup, shift) three times; for a batch
+// the instructions of the chains (half the issue slots, mostly shifts, which
+// issue at half rate).  So a chain's step is branch-free and has two lookups
+// per 32-bit window, every phase runs without divergence, and the groups are
+// dealt out so that the fewest warps do a group more than the others.  Before,
+// a branch per lookup reloaded words from conflicting banks (230 cycles a step
+// against the lookup's 30), the tables came from a launch of their own and a
+// memset, CTA barriers held every warp to the slowest, and the passes kept 36
+// bytes a subsequence instead of 5.  Measured, before and now (768x512, 6,800
+// subsequences an image): 1 image 54.3 -> 24.8 us, 24 images 100.2 -> 45.4 us,
+// 64 images 163 -> 96.5 us; 256 images of 64x64 108 -> 38.4 us.
+#include <algorithm>
 #include <cstdint>
 
 #include <cooperative_groups.h>
@@ -46,80 +65,140 @@ namespace {
 
 constexpr int kQ = PIC_HUFF_WORDS_PER_SUBSEQ;  // words per subsequence
 constexpr int kS = 32 * kQ;                     // bits per subsequence
-constexpr int kThreads = 256;
+// Warps of a CTA: 8, or 9 where that saves a round of groups (24 images of
+// 768x512, 5,129 groups on 152 SMs: 45.4 us in one round, 64 in two).  Nine
+// warps of 56 registers on each of four CTAs fill an SM; ten, at 48
+// registers, spill (69 us).  Fewer than 8 make the tables too slowly (one
+// image: 33 us with 2, 26.9 with 4, 25.9 with 8).
+constexpr int kMaxWarps = 9;
+constexpr int kMinWarps = 8;
+constexpr int kCtasPerSm = 4;
+constexpr int kMaxParts = 8;  // CTAs that share one image's tables (one 100x100 image: 27.0 us with 1, 22.4 with 8)
 constexpr int kMaxPasses = 64;
+constexpr int kHead = 16 + 4 * 68;  // workspace bytes before block_sum (a multiple of 16)
+static_assert(kHead >= 16 + 4 * kMaxPasses && kHead % 16 == 0, "status, pass counters");
 constexpr int kMaxTable = 4096;
 constexpr int kMaxGrid = 8192;
-constexpr int kWbuf = kThreads * kQ + 2;  // stream words of one pass of 256 subsequences
-constexpr int kRound = 16;                // symbols a thread decodes between two warp stores
-constexpr int kRow = kRound + 1;          // staging row (padded against bank conflicts)
-constexpr int kStageInts = kThreads * kRow;
+constexpr int kWords = 32 * kQ + 2;                  // stream words of a warp's 32 subsequences (two past the last)
+constexpr int kWrow = kQ + 1;                        // a subsequence's staged words, and the one that follows
+constexpr int kWbuf = 32 * kWrow + 2;
+constexpr int kRound = 32;                           // symbols a thread decodes between two warp stores
+constexpr int kStep = 8;                             // symbols between two looks at whether any thread goes on
+constexpr int kRow = kRound + 2;                     // staging row, 16-bit entries (odd number of words)
 enum : int { kBadCode = 1, kBadCount = 2, kNoSync = 4, kBadTable = 8 };
 
 struct Ws {
   int* status;           // [4]
   int* changed;          // [kMaxPasses]
-  long long* block_sum;  // [kMaxGrid]
+  long long* block_sum;  // [kMaxGrid]: codewords of each CTA's range
   uint16_t* lut;         // [B][2^p]
-  long long* exit0;      // [n_sub]
-  long long* exit1;      // [n_sub]
-  long long* start;      // [n_sub]
-  long long* off;        // [n_sub]
-  int* cnt;              // [n_sub]
+  uint16_t* cnt;         // [n_sub]: codewords
+  uint8_t* multi;        // [B][2^p]: codewords inside the window << 4 | their bits
+  uint8_t* over0;        // [n_sub]: overshoot, double-buffered over the passes
+  uint8_t* over1;        // [n_sub]
+  uint8_t* start;        // [n_sub]: the overshoot it was decoded from
+  uint8_t* direct;       // [B]: the lookup table holds values, not rows
 };
 
-long long ws_size(long long n_sub, int B, int p) {
-  long long b = 16 + kMaxPasses * 4 + kMaxGrid * 8;
-  b += (static_cast<long long>(B) << p) * 2;
-  b = (b + 15) / 16 * 16;
-  b += n_sub * (8 * 4 + 4);
-  return (b + 15) / 16 * 16;
-}
-
-__host__ __device__ inline Ws ws_view(void* w, long long n_sub, int B, int p) {
+__host__ __device__ inline Ws ws_view(void* w, long long n_sub, int B, int p, long long* bytes = nullptr) {
   char* c = static_cast<char*>(w);
+  const long long tab = static_cast<long long>(B) << p;
   Ws v;
   v.status = reinterpret_cast<int*>(c);
   v.changed = reinterpret_cast<int*>(c + 16);
-  v.block_sum = reinterpret_cast<long long*>(c + 16 + kMaxPasses * 4);
-  v.lut = reinterpret_cast<uint16_t*>(c + 16 + kMaxPasses * 4 + kMaxGrid * 8);
-  long long o = 16 + kMaxPasses * 4 + kMaxGrid * 8 + (static_cast<long long>(B) << p) * 2;
+  v.block_sum = reinterpret_cast<long long*>(c + kHead);
+  long long o = kHead + kMaxGrid * 8;
+  v.lut = reinterpret_cast<uint16_t*>(c + o);
+  o += tab * 2;
+  v.cnt = reinterpret_cast<uint16_t*>(c + o);
+  o += (n_sub * 2 + 15) / 16 * 16;
   o = (o + 15) / 16 * 16;
-  v.exit0 = reinterpret_cast<long long*>(c + o);
-  v.exit1 = v.exit0 + n_sub;
-  v.start = v.exit1 + n_sub;
-  v.off = v.start + n_sub;
-  v.cnt = reinterpret_cast<int*>(v.off + n_sub);
+  v.multi = reinterpret_cast<uint8_t*>(c + o);
+  o += tab;
+  v.over0 = reinterpret_cast<uint8_t*>(c + o);
+  v.over1 = v.over0 + n_sub;
+  v.start = v.over1 + n_sub;
+  v.direct = v.start + n_sub;
+  o += 3 * n_sub + B;
+  if (bytes) *bytes = (o + 15) / 16 * 16;
   return v;
 }
 
-// ---------------------------------------------------------------- 1. tables
-__global__ void __launch_bounds__(kThreads)
-    huff_lut(const int32_t* __restrict__ tab_len, int max_table, int p, uint16_t* lut, int* status) {
-  __shared__ int s_start[kMaxTable + 1];
-  __shared__ uint16_t s_entry[kMaxTable];
-  __shared__ int s_warp[kThreads / 32];
+long long ws_size(long long n_sub, int B, int p) {
+  long long b = 0;
+  ws_view(nullptr, n_sub, B, p, &b);
+  return b;
+}
+
+struct DecodeParams {
+  const uint32_t* words;
+  long long n_words;
+  const long long* word_off;
+  const long long* n_bits;
+  int B;
+  int p;
+  const long long* sym_off;
+  const int32_t* tab_value;  // [B][max_table]: a table entry's low 12 bits index its row
+  const int32_t* tab_len;    // [B][max_table]
+  int max_table;
+  int32_t* out;
+  Ws ws;
+  long long n_sub;
+  // groups of 32 subsequences, dealt out to the CTAs in contiguous ranges
+  // (groups_base each, the first groups_more CTAs one more), and there to the warps
+  long long groups_base;
+  int groups_more;
+  int parts;            // CTAs that share the making of one image's tables
+};
+
+// Dynamic shared memory: two images' tables, the warps' words,
+// staging rows and row descriptors.  (Phase 0 works in the same memory: run starts, then a table.)
+__host__ __device__ constexpr size_t smem_bytes(int p, int warps) {
+  return (size_t{2} * 3 << p) + 16 + size_t(warps) * (4 * (kWbuf + 32) + 2 * 32 * kRow);
+}
+
+__device__ __forceinline__ uint32_t* words_of(uint8_t* s_dyn, int p) {
+  return reinterpret_cast<uint32_t*>(s_dyn + (((size_t{6} << p) + 4 + 15) & ~size_t{15}));
+}
+
+// ---------------------------------------------------------------- 0. tables
+// The part-th of P.parts pieces of image b's lookup and multi tables -> global
+// memory (the whole CTA; the pieces' run starts are worked out by each, the
+// windows' codewords, three quarters of the time, only for the piece).
+// Returns true if the stored table is bad (then every entry is "no codeword").
+__device__ bool build_tables(const DecodeParams& P, int b, int part, void* scratch) {
+  __shared__ int s_warp[kMaxWarps];
   __shared__ int s_m;
-  const int b = blockIdx.x, t = threadIdx.x, lane = t & 31, warp = t >> 5;
-  const int32_t* tl = tab_len + static_cast<long long>(b) * max_table;
+  const int p = P.p, size = 1 << p;
+  uint32_t* s_start = static_cast<uint32_t*>(scratch);                // [2^p + 1]: value << 16 | run start
+  uint16_t* s_lut = reinterpret_cast<uint16_t*>(s_start + size + 1);  // [2^p]
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5, n_threads = blockDim.x, n_warps = n_threads >> 5;
+  const int32_t* tl = P.tab_len + static_cast<long long>(b) * P.max_table;
+  const int32_t* tv = P.tab_value + static_cast<long long>(b) * P.max_table;
   // the table ends at its first zero length
-  if (t == 0) s_m = max_table;
+  __syncthreads();  // (the memory and s_m are free)
+  if (t == 0) s_m = P.max_table;
   __syncthreads();
-  for (int k = t; k < max_table; k += blockDim.x)
-    if (tl[k] == 0) atomicMin(&s_m, k);
-  __syncthreads();
+  bool wide = false;  // values past 12 bits (or such rows behind the table's end: then it is read like one that has)
+#pragma unroll 2
+  for (int k = t; k < P.max_table; k += n_threads) {
+    const int l = __ldg(tl + k), v = __ldg(tv + k);
+    if (l == 0) atomicMin(&s_m, k);
+    wide |= v < -2048 || v > 2047;
+  }
+  const bool direct = !__syncthreads_or(wide);
   const int m = s_m;
-  // run sizes 2^(p - len) scanned into run starts, 256 entries at a time
-  bool bad = false;
+  // run sizes 2^(p - len) scanned into run starts, 256 entries at a time; more
+  // than 2^p entries cannot be a code
+  bool bad = m > size;
   int carry = 0;
-  for (int k0 = 0; k0 < m; k0 += kThreads) {
+  for (int k0 = 0; k0 < m && m <= size; k0 += n_threads) {
     const int k = k0 + t;
     int run = 0;
     if (k < m) {
-      const int l = tl[k];
+      const int l = __ldg(tl + k);
       if (l < 1 || l > p) bad = true;
       else run = 1 << (p - l);
-      s_entry[k] = static_cast<uint16_t>((l << 12) | k);  // the value is tab_value[k]
     }
     int x = run;  // inclusive warp scan, then across the warps
 #pragma unroll
@@ -130,58 +209,75 @@ __global__ void __launch_bounds__(kThreads)
     if (lane == 31) s_warp[warp] = x;
     __syncthreads();
     int before = 0, total = 0;
-    for (int i = 0; i < kThreads / 32; ++i) {
+#pragma unroll
+    for (int i = 0; i < kMaxWarps; ++i) {
+      if (i >= n_warps) break;
       before += i < warp ? s_warp[i] : 0;
       total += s_warp[i];
     }
-    if (k < m) s_start[k] = min(carry + before + x - run, 1 << p);
-    carry = min(carry + total, (1 << p) + 1);  // capped: runs may sum past 2^p only in bad tables
+    if (k < m) {
+      s_start[k] = static_cast<uint32_t>(__ldg(tv + k)) << 16 | static_cast<uint32_t>(min(carry + before + x - run, size));
+    }
+    carry = min(carry + total, size + 1);  // capped: runs may sum past 2^p only in bad tables
     __syncthreads();
   }
-  bad = __syncthreads_or(bad) || carry > (1 << p);  // a bad length, or Kraft's inequality violated
-  if (t == 0) {
-    s_start[m] = bad ? 0 : carry;
-    if (bad) atomicOr(status, kBadTable);
-  }
+  bad = __syncthreads_or(bad) || carry > size;  // a bad length, or Kraft's inequality violated
+  const int fill = bad ? 0 : carry;  // a bad table decodes nothing
+  if (t == 0 && m <= size) s_start[m] = fill;
+  if (t == 0) P.ws.direct[b] = direct;
   __syncthreads();
-  const int fill = s_start[m];  // a bad table decodes nothing: every entry "no codeword"
-  uint16_t* out = lut + (static_cast<long long>(b) << p);
-  // every entry finds its run by binary search over the run starts
-  for (int i = t; i < (1 << p); i += blockDim.x) {
-    uint16_t e = 0;  // no codeword
-    if (i < fill) {
-      int lo = 0, hi = m - 1;  // last k with s_start[k] <= i
+  auto entry = [&](int k, int& next) {  // and where symbol k's run ends
+    const uint32_t v = s_start[k];
+    next = s_start[k + 1] & 0xFFFF;
+    const int len = p - (31 - __clz(next - static_cast<int>(v & 0xFFFF)));
+    return static_cast<int>((direct ? v >> 16 : static_cast<uint32_t>(k)) << 4) | len;
+  };
+  // each thread finds the run of its first entry and walks on from there
+  const int per = (size + n_threads - 1) / n_threads;
+  uint16_t* lut = P.ws.lut + (static_cast<long long>(b) << p);
+  uint8_t* multi = P.ws.multi + (static_cast<long long>(b) << p);
+  const int i0 = t * per;
+  if (i0 < size) {
+    int lo = 0, e = 0, next = 0;
+    if (i0 < fill) {
+      int hi = m - 1;  // last k with s_start[k] <= i0
       while (lo < hi) {
         const int mid = (lo + hi + 1) >> 1;
-        if (s_start[mid] <= i) lo = mid;
+        if (static_cast<int>(s_start[mid] & 0xFFFF) <= i0) lo = mid;
         else hi = mid - 1;
       }
-      e = s_entry[lo];
+      e = entry(lo, next);
     }
-    out[i] = e;
+    for (int i = i0; i < min(i0 + per, size); ++i) {
+      if (i >= fill) {
+        e = 0;  // no codeword
+      } else if (i >= next) {
+        e = entry(++lo, next);
+      }
+      s_lut[i] = static_cast<uint16_t>(e);
+    }
   }
+  __syncthreads();
+  const int piece = size / P.parts;
+  for (int i = part * piece + t; i < (part + 1) * piece; i += n_threads) {
+    lut[i] = s_lut[i];
+    int pos = 0, c = 0;
+    while (pos < p) {
+      const int l = s_lut[(i << pos) & (size - 1)] & 15;
+      if (l == 0 || pos + l > p) break;
+      pos += l;
+      ++c;
+    }
+    if (c == 0) c = pos = 1;  // no codeword: counted as one of 1 bit (the final decode reports it)
+    multi[i] = static_cast<uint8_t>((c << 4) | pos);
+  }
+  return bad;
 }
 
-// --------------------------------------------------------------- 2. decode
-struct DecodeParams {
-  const uint32_t* words;
-  long long n_words;
-  const long long* word_off;
-  const long long* n_bits;
-  int B;
-  int p;
-  const long long* sym_off;
-  const int32_t* tab_value;  // [B][max_table]: a table entry's low 12 bits index its row
-  int max_table;
-  int32_t* out;
-  Ws ws;
-  long long n_sub;
-  long long per_block;  // subsequences per CTA, a multiple of kThreads
-};
-
-__device__ __forceinline__ int image_of(const DecodeParams& P, long long word) {
-  int lo = 0, hi = P.B - 1;  // last b with word_off[b] <= word
-  while (lo < hi) {
+// --------------------------------------------------------------- 1. decode
+// The image of stream word `word`, among images lo .. hi.
+__device__ __forceinline__ int image_of(const DecodeParams& P, long long word, int lo, int hi) {
+  while (lo < hi) {  // last b with word_off[b] <= word
     const int mid = (lo + hi + 1) >> 1;
     if (__ldg(P.word_off + mid) <= word) lo = mid;
     else hi = mid - 1;
@@ -189,77 +285,77 @@ __device__ __forceinline__ int image_of(const DecodeParams& P, long long word) {
   return lo;
 }
 
-// The counting loop of decode_span_s, with (PAIR) or without the pair table.
-template <bool PAIR>
-__device__ __forceinline__ int decode_span_loop(const uint32_t* sw, int lpos, int lke, const uint16_t* lut,
-                                                const uint8_t* lut2, int p, int* count, bool* bad) {
-  int c = 0;
-  int li = lpos >> 5;
-  uint32_t hi = sw[li], lo = sw[li + 1];
-  const int shr = 32 - p;
-  while (lpos < lke) {
-    const int wi = lpos >> 5;
-    if (wi != li) {  // crossed into the next word (a step covers at most p <= 12 bits)
-      li = wi;
-      hi = lo;
-      lo = sw[li + 1];
+// An image's tables for the decode loops: in shared memory (SH), or in global
+// memory for the images that lie strictly inside a CTA's range.
+template <bool SH>
+struct Tables {
+  uint32_t lut_s, multi_s;  // shared addresses
+  const uint16_t* lut_g;
+  const uint8_t* multi_g;
+  __device__ __forceinline__ int lut(uint32_t w) const {
+    if (SH) {
+      unsigned short v;
+      asm volatile("ld.shared.u16 %0, [%1];" : "=h"(v) : "r"(lut_s + 2 * w));
+      return v;
     }
-    const uint32_t w = __funnelshift_l(lo, hi, lpos & 31) >> shr;
-    if constexpr (PAIR) {
-      const uint32_t e2 = lut2[w];
-      int l1 = static_cast<int>(e2 & 15u);
-      const int l2 = static_cast<int>(e2 >> 4);
-      if (l1 == 0) {
-        *bad = true;
-        l1 = 1;
+    return lut_g[w];
+  }
+  __device__ __forceinline__ int multi(uint32_t w) const {
+    if (SH) {
+      unsigned short v;
+      asm volatile("{\n\t.reg .b32 t;\n\tld.shared.u8 t, [%1];\n\tcvt.u16.u32 %0, t;\n\t}" : "=h"(v) : "r"(multi_s + w));
+      return v;
+    }
+    return multi_g[w];
+  }
+};
+
+// The 32 bits at bit `pos` of a subsequence's staged words: two codewords.
+__device__ __forceinline__ uint32_t window(const uint32_t* row, int pos) {
+  const uint32_t* w = row + (pos >> 5);
+  return __funnelshift_l(w[1], w[0], pos);
+}
+
+// Counts the codewords that start at bits pos .. end - 1 of a subsequence's
+// staged words, the first at pos; pos becomes the first codeword boundary at
+// or after end.  The whole warp goes through it together, without divergence;
+// lanes with pos >= end take no part.
+template <bool SH>
+__device__ __forceinline__ int count_span(const uint32_t* row, int& pos, int end, const Tables<SH>& tab, int p) {
+  const int shr = 32 - p, begin = pos;
+  int sum = 0;  // of the windows' entries: 16 x codewords + bits
+  // whole windows: every codeword inside one that ends by `end` starts before it
+  while (__any_sync(0xffffffffu, pos + p <= end)) {
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      const uint32_t w = window(row, pos);
+      const int e0 = tab.multi(w >> shr);
+      const int e1 = tab.multi(w << (e0 & 15) >> shr);
+      if (pos + p <= end) {
+        sum += e0;
+        pos += e0 & 15;
       }
-      const bool two = l2 != 0 && lpos + l1 < lke;
-      c += two ? 2 : 1;
-      lpos += two ? l1 + l2 : l1;
-    } else {
-      int len = static_cast<int>(lut[w] >> 12);
-      if (len == 0) {
-        *bad = true;
-        len = 1;
+      if (pos + p <= end) {
+        sum += e1;
+        pos += e1 & 15;
       }
+    }
+  }
+  int c = (sum - (pos - begin)) >> 4;
+  while (__any_sync(0xffffffffu, pos < end)) {
+    const uint32_t w = window(row, pos);
+    const int l0 = max(tab.lut(w >> shr) & 15, 1);
+    const int l1 = max(tab.lut(w << l0 >> shr) & 15, 1);
+    if (pos < end) {
       ++c;
-      lpos += len;
+      pos += l0;
+    }
+    if (pos < end) {
+      ++c;
+      pos += l1;
     }
   }
-  *count = c;
-  return lpos;
-}
-
-// Counts the codewords from bit `lpos` of the words staged in shared memory
-// (bit 0 = the top bit of sw[0]) while lpos < lke; returns the position
-// after the last codeword.  *bad is raised on a bit pattern that is no
-// codeword.  The next p bits come from one funnel shift of the two current
-// words.  With a pair table (lut2: the lengths of the first codeword of each
-// p-bit window and of the second one when it lies inside the same window),
-// one lookup advances over up to two codewords.
-__device__ __forceinline__ int decode_span_s(const uint32_t* sw, int lpos, int lke, const uint16_t* lut,
-                                             const uint8_t* lut2, int p, int* count, bool* bad) {
-  if (lpos >= lke) {
-    *count = 0;
-    return lpos;
-  }
-  return lut2 ? decode_span_loop<true>(sw, lpos, lke, lut, lut2, p, count, bad)
-              : decode_span_loop<false>(sw, lpos, lke, lut, lut2, p, count, bad);
-}
-
-// decode_span_s for subsequence positions of image b: pos (bits from the
-// image's first word wbase) <-> staged position (bits from word w0).
-__device__ __forceinline__ long long decode_at(const uint32_t* sw, long long w0, long long wbase, long long pos,
-                                               long long ke, const uint16_t* lut, const uint8_t* lut2, int p,
-                                               int* count, bool* bad) {
-  if (pos >= ke) {
-    *count = 0;
-    return pos;
-  }
-  const long long shift = (wbase - w0) * 32;  // staged bit = image bit + shift (>= 0 here)
-  const int lp = decode_span_s(sw, static_cast<int>(pos + shift), static_cast<int>(ke + shift), lut, lut2, p,
-                               count, bad);
-  return lp - shift;
+  return c;
 }
 
 __device__ long long block_sum_ll(long long v, long long* red) {
@@ -270,251 +366,307 @@ __device__ long long block_sum_ll(long long v, long long* red) {
   if (lane == 0) red[warp] = v;
   __syncthreads();
   long long t = 0;
-  for (int i = 0; i < kThreads / 32; ++i) t += red[i];
+#pragma unroll
+  for (int i = 0; i < kMaxWarps; ++i) t += i < static_cast<int>(blockDim.x >> 5) ? red[i] : 0;
   return t;
 }
 
-__global__ void __launch_bounds__(kThreads) huff_decode(const DecodeParams P) {
-  cg::grid_group grid = cg::this_grid();
-  __shared__ long long red[kThreads / 32];
-  __shared__ long long scan[kThreads];
-  extern __shared__ __align__(16) uint32_t s_dyn[];
-  uint16_t* s_lut = reinterpret_cast<uint16_t*>(s_dyn);  // tables of the first and last image of the range
-  const Ws& ws = P.ws;
-  const long long per_block = P.per_block;
-  const long long k_begin = static_cast<long long>(blockIdx.x) * per_block;
-  const long long k_end = min(k_begin + per_block, P.n_sub);
-  bool bad = false;
-  // every lookup is a dependent load in a decode chain: the CTA's images'
-  // tables go to shared memory (images between the first and the last of
-  // the range, which only tiny streams produce, read theirs from global)
-  const int tsize = 1 << P.p;
-  const int b_first = k_begin < k_end ? image_of(P, k_begin * kQ) : 0;
-  const int b_last = k_begin < k_end ? image_of(P, (k_end - 1) * kQ) : 0;
-  for (int i = threadIdx.x; i < tsize; i += blockDim.x) {
-    s_lut[i] = ws.lut[(static_cast<long long>(b_first) << P.p) + i];
-    s_lut[tsize + i] = ws.lut[(static_cast<long long>(b_last) << P.p) + i];
-  }
-  __syncthreads();
-  auto lut_of = [&](int b) -> const uint16_t* {
-    return b == b_first ? s_lut : (b == b_last ? s_lut + tsize : ws.lut + (static_cast<long long>(b) << P.p));
-  };
-  // each pass of 256 subsequences first stages its stream words (coalesced),
-  // so that no global load sits inside a decode chain
-  uint32_t* s_words = reinterpret_cast<uint32_t*>(s_lut + 2 * tsize);
-  int* s_stage = reinterpret_cast<int*>(s_words + kWbuf);
-  // the pair tables of the two images: first codeword's length | the
-  // second's << 4 (0 when it does not lie inside the same p-bit window)
-  uint8_t* s_lut2 = reinterpret_cast<uint8_t*>(s_stage + kStageInts);
-  for (int i = threadIdx.x; i < 2 * tsize; i += blockDim.x) {
-    const uint16_t* L = s_lut + (i >= tsize ? tsize : 0);
-    const int w = i & (tsize - 1);
-    const int l1 = static_cast<int>(L[w] >> 12);
-    int l2 = 0;
-    if (l1 > 0 && l1 < P.p) {
-      const int l = static_cast<int>(L[(w << l1) & (tsize - 1)] >> 12);
-      if (l > 0 && l <= P.p - l1) l2 = l;
+// 32 subsequences' stream words -> shared memory (a warp; coalesced), so that
+// no global load sits inside a decode chain.
+__device__ __forceinline__ void stage(const DecodeParams& P, uint32_t* s_words, long long k0) {
+  const int lane = threadIdx.x & 31;
+  const long long w0 = k0 * kQ;
+#pragma unroll
+  for (int j = 0; j < (kWords + 31) / 32; ++j) {
+    const int i = lane + 32 * j, at = i + i / kQ;
+    if (i < kWords) {
+      const uint32_t w = w0 + i < P.n_words ? __ldg(P.words + w0 + i) : 0u;
+      s_words[at] = w;
+      if (i % kQ == 0 && i > 0) s_words[at - 1] = w;
     }
-    s_lut2[i] = static_cast<uint8_t>(l1 | (l2 << 4));
   }
-  __syncthreads();
-  auto lut2_of = [&](int b) -> const uint8_t* {
-    return b == b_first ? s_lut2 : (b == b_last ? s_lut2 + tsize : nullptr);
+}
+
+// Phases a to d, with every image's tables in shared memory (SH) or not, for
+// subsequences [k_begin, k_end) of this warp.
+template <bool SH>
+__device__ __forceinline__ void decode_phases(const DecodeParams& P, cg::grid_group& grid, uint8_t* s_dyn, int b_first,
+                                              int b_last, long long k_begin, long long k_end) {
+  __shared__ long long red[kMaxWarps];
+  __shared__ long long wsum[kMaxWarps];
+  const Ws& ws = P.ws;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, size = 1 << P.p;
+  const int n_threads = blockDim.x, n_warps = n_threads >> 5;
+  uint32_t* const all_words = words_of(s_dyn, P.p);
+  uint32_t* const s_words = all_words + warp * kWbuf;
+  uint32_t* const s_desc = all_words + n_warps * kWbuf + warp * 32;
+  uint16_t* const wbuf = reinterpret_cast<uint16_t*>(all_words + n_warps * (kWbuf + 32)) + warp * 32 * kRow;
+  const uint32_t lut_s = static_cast<uint32_t>(__cvta_generic_to_shared(s_dyn)), multi_s = lut_s + 4 * size;
+  auto tables = [&](int b) {
+    Tables<SH> t;
+    if (SH) {
+      t.lut_s = lut_s + (b == b_first ? 0 : 2 * size);
+      t.multi_s = multi_s + (b == b_first ? 0 : size);
+    } else {
+      t.lut_g = ws.lut + (static_cast<long long>(b) << P.p);
+      t.multi_g = ws.multi + (static_cast<long long>(b) << P.p);
+    }
+    return t;
   };
+  long long held = k_begin;  // first subsequence of the words held: staged before the tables were made
   auto stage_words = [&](long long k0) {
-    const long long w0 = k0 * kQ;
-    __syncthreads();
-    for (int i = threadIdx.x; i < kWbuf; i += blockDim.x)
-      s_words[i] = w0 + i < P.n_words ? __ldg(P.words + w0 + i) : 0u;
-    __syncthreads();
+    if (k0 == held) return;
+    held = k0;
+    __syncwarp();  // the words before have been read
+    stage(P, s_words, k0);
+    __syncwarp();
   };
+  // Subsequence k: its image, whether it is the image's first or last, its
+  // bits (0: past the image's last bit).
+  auto locate = [&](long long k, int& b, bool& first, bool& last) -> int {
+    b = image_of(P, k * kQ, b_first, b_last);
+    const long long ks = (k * kQ - __ldg(P.word_off + b)) * 32, left = __ldg(P.n_bits + b) - ks;
+    first = ks == 0;
+    last = left <= kS;
+    return static_cast<int>(max(min(static_cast<long long>(kS), left), 0LL));
+  };
+  const uint32_t* const row = s_words + lane * kWrow;  // this lane's subsequence
 
   // a. speculative decode of every subsequence from its first bit
-  for (long long k0 = k_begin; k0 < k_end; k0 += kThreads) {
+  for (long long k0 = k_begin; k0 < k_end; k0 += 32) {
     stage_words(k0);
-    const long long k = k0 + threadIdx.x;
-    if (k >= k_end) continue;
-    const int b = image_of(P, k * kQ);
-    const long long wbase = __ldg(P.word_off + b), nb = __ldg(P.n_bits + b);
-    const long long ks = (k * kQ - wbase) * 32, ke = min(ks + kS, nb);
-    int c = 0;
-    bool junk = false;
-    const long long ex = decode_at(s_words, k0 * kQ, wbase, ks, ke, lut_of(b), lut2_of(b), P.p, &c, &junk);
-    ws.exit0[k] = ex;
-    ws.start[k] = ks;
-    ws.cnt[k] = c;
+    const long long k = k0 + lane;
+    int b = b_first, bits = 0;
+    bool first, last;
+    if (k < k_end) bits = locate(k, b, first, last);
+    int pos = 0;
+    count_span<SH>(row, pos, bits, tables(b), P.p);
+    if (k < k_end) ws.over0[k] = static_cast<uint8_t>(max(pos - kS, 0));
   }
   grid.sync();
 
-  // b. synchronisation passes (exits double-buffered)
-  int pass = 0;
+  // b. synchronisation passes
   bool stable = false;
-  for (; pass < kMaxPasses; ++pass) {
-    const long long* ex_in = (pass & 1) ? ws.exit1 : ws.exit0;
-    long long* ex_out = (pass & 1) ? ws.exit0 : ws.exit1;
-    long long ch = 0;
-    for (long long k0 = k_begin; k0 < k_end; k0 += kThreads) {
-      const long long k = k0 + threadIdx.x;
-      int b = 0;
-      long long wbase = 0, nb = 0, ks = 0, st = 0;
+  for (int pass = 0; pass < kMaxPasses; ++pass) {
+    const uint8_t* in = (pass & 1) ? ws.over1 : ws.over0;
+    uint8_t* out = (pass & 1) ? ws.over0 : ws.over1;
+    bool changed = false;
+    long long total = 0;
+    for (long long k0 = k_begin; k0 < k_end; k0 += 32) {
+      const long long k = k0 + lane;
+      int b = b_first, bits = 0, st = 0, c = 0, over = 0;
       bool redo = false;
       if (k < k_end) {
-        b = image_of(P, k * kQ);
-        wbase = __ldg(P.word_off + b);
-        nb = __ldg(P.n_bits + b);
-        ks = (k * kQ - wbase) * 32;
-        st = ks == 0 || ks >= nb ? ws.start[k] : ex_in[k - 1];
-        redo = st != ws.start[k];
-        if (!redo) ex_out[k] = ex_in[k];
+        bool first, last;
+        bits = locate(k, b, first, last);
+        st = first || bits == 0 || k == 0 ? 0 : __ldcg(in + k - 1);
+        redo = pass == 0 || st != ws.start[k];
+        if (pass > 0) c = ws.cnt[k];
+        over = in[k];
+        if (!redo) out[k] = static_cast<uint8_t>(over);
       }
-      if (!__syncthreads_or(redo)) continue;  // nothing to redo in this pass of the CTA
-      stage_words(k0);
-      if (redo) {
-        int c = 0;
-        bool junk = false;
-        ex_out[k] = decode_at(s_words, k0 * kQ, wbase, st, min(ks + kS, nb), lut_of(b), lut2_of(b), P.p, &c,
-                              &junk);
-        ws.start[k] = st;
-        ws.cnt[k] = c;
-        ++ch;
+      if (__any_sync(0xffffffffu, redo)) {
+        stage_words(k0);
+        int pos = st;
+        const int c_now = count_span<SH>(row, pos, redo ? bits : 0, tables(b), P.p);
+        if (redo) {
+          c = c_now;
+          const int over_now = max(pos - kS, 0);
+          changed |= over_now != over;
+          out[k] = static_cast<uint8_t>(over_now);
+          ws.start[k] = static_cast<uint8_t>(st);
+          ws.cnt[k] = static_cast<uint16_t>(c);
+        }
       }
+      total += c;
     }
-    ch = block_sum_ll(ch, red);
-    if (threadIdx.x == 0 && ch) atomicAdd(ws.changed + pass, 1);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) total += __shfl_xor_sync(0xffffffffu, total, o);
+    if (lane == 0) wsum[warp] = total;
+    if (__syncthreads_or(changed) && tid == 0) atomicAdd(ws.changed + pass, 1);
+    if (tid == 0) {
+      long long all = 0;
+#pragma unroll
+      for (int i = 0; i < kMaxWarps; ++i) all += i < n_warps ? wsum[i] : 0;
+      ws.block_sum[blockIdx.x] = all;
+    }
     grid.sync();
     if (*reinterpret_cast<volatile int*>(ws.changed + pass) == 0) {
       stable = true;
       break;
     }
   }
-  if (!stable && blockIdx.x == 0 && threadIdx.x == 0) atomicOr(ws.status, kNoSync);
+  if (!stable && blockIdx.x == 0 && tid == 0) atomicOr(ws.status, kNoSync);
 
-  // c. output positions: exclusive scan of the counts in subsequence order
-  long long mine = 0;
-  for (long long k = k_begin + threadIdx.x; k < k_end; k += blockDim.x) mine += ws.cnt[k];
-  mine = block_sum_ll(mine, red);
-  if (threadIdx.x == 0) ws.block_sum[blockIdx.x] = mine;
-  grid.sync();
-  long long base = 0;
-  for (int j = threadIdx.x; j < static_cast<int>(blockIdx.x); j += blockDim.x) base += ws.block_sum[j];
-  base = block_sum_ll(base, red);
-  long long carry = base;
-  for (long long k0 = k_begin; k0 < k_end; k0 += blockDim.x) {
-    const long long k = k0 + threadIdx.x;
-    const long long v = k < k_end ? ws.cnt[k] : 0;
-    const int ln = threadIdx.x & 31, wp = threadIdx.x >> 5;
-    long long x = v;  // inclusive scan: warp shuffles, then the warp totals
+  // c. this warp's output position
+  long long carry = 0;
+  for (int j = tid; j < static_cast<int>(blockIdx.x); j += n_threads) carry += __ldcg(ws.block_sum + j);
+  carry = block_sum_ll(carry, red);
+  for (int i = 0; i < warp; ++i) carry += wsum[i];
+
+  // d. final decode from the synchronised starts.  Each lane decodes its
+  // subsequence in rounds of up to kRound symbols into its row of the warp's
+  // buffer; the warp then stores the rows, one per instruction, instead of 32
+  // scattered words.
+  const int shr = 32 - P.p;
+  bool bad = false;
+  for (long long k0 = k_begin; k0 < k_end; k0 += 32) {
+    stage_words(k0);
+    const long long k = k0 + lane;
+    int b = b_first, end = 0, pos = 0, n_mine = 0;
+    bool first = false, last = false;
+    if (k < k_end) {
+      end = locate(k, b, first, last);
+      pos = ws.start[k];
+      n_mine = ws.cnt[k];
+    }
+    const bool some = end > 0;
+    // output positions: exclusive scan of the counts
+    int x = n_mine;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
-      const long long y = __shfl_up_sync(0xffffffffu, x, o);
-      if (ln >= o) x += y;
+      const int y = __shfl_up_sync(0xffffffffu, x, o);
+      if (lane >= o) x += y;
     }
-    __syncthreads();  // scan[] of the previous pass has been read
-    if (ln == 31) scan[wp] = x;
-    __syncthreads();
-    long long before = 0, all = 0;
-#pragma unroll
-    for (int i = 0; i < kThreads / 32; ++i) {
-      before += i < wp ? scan[i] : 0;
-      all += scan[i];
-    }
-    if (k < k_end) ws.off[k] = carry + before + x - v;
-    carry += all;
-  }
-  if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0 && carry != __ldg(P.sym_off + P.B))
-    atomicOr(ws.status, kBadCount);
-  __syncthreads();
-
-  // d. final decode from the synchronised starts.  Each thread decodes its
-  // subsequence in rounds of up to kRound symbols into its row of a per-warp
-  // shared buffer; the warp then stores two threads' rows per instruction
-  // (lanes 0-15 and 16-31: two 64-byte runs) instead of 32 scattered words.
-  int* wbuf = s_stage + (threadIdx.x >> 5) * 32 * kRow;
-  const int lane = threadIdx.x & 31;
-  for (long long k0 = k_begin; k0 < k_end; k0 += kThreads) {
-    stage_words(k0);
-    const long long k = k0 + threadIdx.x;
-    int lpos = 0, lke = 0, li = 0;
-    uint32_t hi = 0, lo = 0;
-    long long o = 0, room = 0, shift = 0, nb = 0, ks = 0;
-    const uint16_t* lut = s_lut;
-    const int32_t* vals = P.tab_value;
-    bool more = false;
+    int32_t* const dst = P.out + carry + lane;
+    int at = x - n_mine;  // this lane's next symbol, from carry on: at most 32 x (256 + kRound)
+    int room = 0;         // and how many it may still write
     if (k < k_end) {
-      const int b = image_of(P, k * kQ);
-      const long long wbase = __ldg(P.word_off + b);
-      nb = __ldg(P.n_bits + b);
-      ks = (k * kQ - wbase) * 32;
-      o = ws.off[k];
-      const long long img_end = __ldg(P.sym_off + b + 1);
-      if (ks == 0 && o != __ldg(P.sym_off + b)) atomicOr(ws.status, kBadCount);
-      room = o < img_end ? img_end - o : 0;
-      shift = (wbase - k0 * kQ) * 32;
-      const long long st = ws.start[k], ke = min(ks + kS, nb);
-      lpos = static_cast<int>(st + shift);
-      lke = static_cast<int>(ke + shift);
-      lut = lut_of(b);
-      vals = P.tab_value + static_cast<long long>(b) * P.max_table;
-      more = ks < nb && st < ke;
-      if (more) {
-        li = lpos >> 5;
-        hi = s_words[li];
-        lo = s_words[li + 1];
-      }
+      const long long o = carry + at, img_end = __ldg(P.sym_off + b + 1);
+      if (first && o != __ldg(P.sym_off + b)) atomicOr(ws.status, kBadCount);
+      room = static_cast<int>(max(min(img_end - o, 1LL << 16), 0LL));
     }
-    const int shr = 32 - P.p;
-    long long done = 0;
-    while (__any_sync(0xffffffffu, more)) {
+    carry += __shfl_sync(0xffffffffu, x, 31);
+    const Tables<SH> tab = tables(b);
+    // this lane's rows in the value table (at most 2^28); -1: its entries are values
+    const int vals = __ldcg(ws.direct + b) ? -1 : b * P.max_table;
+    const bool direct = __all_sync(0xffffffffu, vals < 0);
+    while (__any_sync(0xffffffffu, pos < end)) {
       int n = 0;
-      while (more && n < kRound) {
-        const int wi = lpos >> 5;
-        if (wi != li) {
-          li = wi;
-          hi = lo;
-          lo = s_words[li + 1];
+#pragma unroll
+      for (int u0 = 0; u0 < kRound; u0 += kStep) {
+        int len = 1;
+#pragma unroll
+        for (int u = u0; u < u0 + kStep; u += 2) {  // the whole warp, without divergence
+          const uint32_t w = window(row, pos);
+          const int e0 = tab.lut(w >> shr), l0 = e0 & 15;
+          const int e1 = tab.lut(w << l0 >> shr);
+          len = e1 & 15;
+          wbuf[lane * kRow + u] = static_cast<uint16_t>(e0);
+          wbuf[lane * kRow + u + 1] = static_cast<uint16_t>(e1);
+          if (pos < end) {
+            pos += l0;
+            ++n;
+          }
+          if (pos < end) {
+            pos += len;
+            ++n;
+          }
         }
-        const uint32_t e = lut[__funnelshift_l(lo, hi, lpos & 31) >> shr];
-        int len = static_cast<int>(e >> 12);
-        if (len == 0) {
+        if (len == 0 && pos < end) {  // stuck at a bit pattern that is no codeword
           bad = true;
-          len = 1;
+          pos = end;
         }
-        wbuf[lane * kRow + n] = __ldg(vals + (e & 0xFFFu));  // off the decode chain
-        ++n;
-        lpos += len;
-        more = lpos < lke;
+        if (!__any_sync(0xffffffffu, pos < end)) break;
       }
+      // one word describes a lane's row: where it goes, and how much of it
+      s_desc[lane] = static_cast<unsigned>(at) << 6 | static_cast<unsigned>(max(min(n, room), 0));
+      at += n;
+      room -= n;  // (negative: more symbols than the image has)
       __syncwarp();
-      // this thread's output run: cap values at o + done.  Lanes hold
-      // consecutive subsequences, so o + done never falls below lane 0's and
-      // exceeds it by less than 2^13 (32 subsequences of at most 256
-      // codewords): one shuffle per row carries (offset from lane 0, cap).
-      const long long left = room - done;  // symbols this thread may still write
-      const int cap = static_cast<int>(min(static_cast<long long>(n), max(left, 0LL)));
-      const long long at0 = __shfl_sync(0xffffffffu, o + done, 0);
-      const unsigned packed = (static_cast<unsigned>(o + done - at0) << 5) | static_cast<unsigned>(cap);
-#pragma unroll 4
-      for (int j = 0; j < 16; ++j) {
-        const int src = 2 * j + (lane >> 4), i = lane & 15;
-        const unsigned pk = __shfl_sync(0xffffffffu, packed, src);
-        if (i < static_cast<int>(pk & 31u)) P.out[at0 + (pk >> 5) + i] = wbuf[src * kRow + i];
+      // eight rows' loads ahead of their stores (which the compiler cannot
+      // tell from the shared memory they come from)
+#pragma unroll
+      for (int j0 = 0; j0 < 32; j0 += 8) {
+        unsigned pk[8];
+        int q[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+          pk[j] = s_desc[j0 + j];
+          q[j] = static_cast<int16_t>(wbuf[(j0 + j) * kRow + lane]) >> 4;
+        }
+        if (!direct) {
+#pragma unroll
+          for (int j = 0; j < 8; ++j) {
+            const int v = __shfl_sync(0xffffffffu, vals, j0 + j);
+            if (v >= 0 && lane < static_cast<int>(pk[j] & 63u)) q[j] = __ldg(P.tab_value + v + (q[j] & 0xFFF));
+          }
+        }
+#pragma unroll
+        for (int j = 0; j < 8; ++j)
+          if (lane < static_cast<int>(pk[j] & 63u)) dst[pk[j] >> 6] = q[j];
       }
-      done += n;
       __syncwarp();
     }
-    if (k < k_end && ks < nb) {
-      if (done > room) atomicOr(ws.status, kBadCount);
-      if (ks + kS >= nb && lpos - shift != nb) atomicOr(ws.status, kBadCode);  // the last codeword overruns
+    if (some) {
+      if (room < 0) atomicOr(ws.status, kBadCount);
+      if (last && pos != end) atomicOr(ws.status, kBadCode);  // the image's last codeword overruns
     }
   }
+  if (blockIdx.x == gridDim.x - 1 && tid == n_threads - 1 && carry != __ldg(P.sym_off + P.B))
+    atomicOr(ws.status, kBadCount);
   if (bad) atomicOr(ws.status, kBadCode);
+}
+
+__global__ void __launch_bounds__(kMaxWarps * 32, kCtasPerSm) huff_decode(const DecodeParams P) {
+  cg::grid_group grid = cg::this_grid();
+  extern __shared__ __align__(16) uint8_t s_dyn[];
+  const Ws& ws = P.ws;
+  const int tid = threadIdx.x, n_threads = blockDim.x, n_warps = n_threads >> 5;
+
+  // this CTA's groups, and this warp's among them
+  const int cta = blockIdx.x, warp = tid >> 5;
+  const long long g_cta = P.groups_base + (cta < P.groups_more), g0 = cta * P.groups_base + min(cta, P.groups_more);
+  const int g_warp = static_cast<int>(g_cta / n_warps), g_more = static_cast<int>(g_cta % n_warps);
+  const long long gw = g0 + warp * static_cast<long long>(g_warp) + min(warp, g_more);
+  const long long c_begin = min(32 * g0, P.n_sub), c_end = min(32 * (g0 + g_cta), P.n_sub);
+  const long long k_begin = min(32 * gw, P.n_sub), k_end = min(32 * (gw + g_warp + (warp < g_more)), P.n_sub);
+  // the first words, which the making of the tables leaves alone
+  stage(P, words_of(s_dyn, P.p) + (tid >> 5) * kWbuf, k_begin);
+
+  // 0. tables
+  if (blockIdx.x == 0 && tid < 4 + kMaxPasses) ws.status[tid] = 0;  // and the pass counters behind it
+  bool bad_table = false;
+  for (int u = blockIdx.x; u < P.B * P.parts; u += gridDim.x)
+    bad_table |= build_tables(P, u / P.parts, u % P.parts, s_dyn);
+  grid.sync();
+  if (bad_table && tid == 0) atomicOr(ws.status, kBadTable);
+
+  // every lookup is a dependent load in a decode chain: the tables of the
+  // CTA's first and last image go to shared memory.  A range with images in
+  // between (only tiny streams produce one) reads all of its from global.
+  const int size = 1 << P.p;
+  const int b_first = image_of(P, c_begin * kQ, 0, P.B - 1);
+  const int b_last = image_of(P, (c_end - 1) * kQ, b_first, P.B - 1);
+  if (b_last - b_first > 1) {
+    decode_phases<false>(P, grid, s_dyn, b_first, b_last, k_begin, k_end);
+    return;
+  }
+  for (int q = 0; q <= b_last - b_first; ++q) {
+    const uint16_t* gl = ws.lut + (static_cast<long long>(b_first + q) << P.p);
+    const uint8_t* gm = ws.multi + (static_cast<long long>(b_first + q) << P.p);
+    uint8_t* sl = s_dyn + q * 2 * size;
+    uint8_t* sm = s_dyn + (4 + q) * size;
+    if (P.p >= 4) {
+#pragma unroll 2
+      for (int i = tid; i < size / 8; i += n_threads)
+        reinterpret_cast<uint4*>(sl)[i] = __ldcg(reinterpret_cast<const uint4*>(gl) + i);
+      for (int i = tid; i < size / 16; i += n_threads)
+        reinterpret_cast<uint4*>(sm)[i] = __ldcg(reinterpret_cast<const uint4*>(gm) + i);
+    } else if (tid < size) {
+      reinterpret_cast<uint16_t*>(sl)[tid] = __ldcg(gl + tid);
+      sm[tid] = __ldcg(gm + tid);
+    }
+  }
+  __syncthreads();
+  decode_phases<true>(P, grid, s_dyn, b_first, b_last, k_begin, k_end);
 }
 
 bool aligned(const void* p, uintptr_t a) { return (reinterpret_cast<uintptr_t>(p) % a) == 0; }
 
 // Resident CTAs of huff_decode on the current device with `smem` bytes of
 // lookup tables each (the cooperative grid), per device and precision.
-int decode_grid(int p, size_t smem, int* grid) {
+int decode_grid(int p, int* grid) {
   constexpr int kMaxDev = 64;
   static int cached[kMaxDev][PIC_HUFF_MAX_PRECISION + 1];
   int dev = 0;
@@ -525,12 +677,13 @@ int decode_grid(int p, size_t smem, int* grid) {
   if (cached[dev][p] == 0) {
     int coop = 0, sms = 0, per_sm = 0;
     // the attribute is the function's, for every precision: set it to the largest
-    constexpr int kMaxSmem = (3 * 2 << PIC_HUFF_MAX_PRECISION) + (kWbuf + kStageInts) * 4;
-    if (cudaFuncSetAttribute(huff_decode, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem) !=
+    if (cudaFuncSetAttribute(huff_decode, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             static_cast<int>(smem_bytes(PIC_HUFF_MAX_PRECISION, kMaxWarps))) !=
             cudaSuccess ||
         cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, huff_decode, kThreads, smem) != cudaSuccess) {
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, huff_decode, 32 * kMaxWarps,
+                                                      smem_bytes(p, kMaxWarps)) != cudaSuccess) {
       cudaGetLastError();
       return PIC_ERR_CUDA;
     }
@@ -563,10 +716,8 @@ int pic_huffman_decode(const uint32_t* words, int64_t n_words, const int64_t* wo
     return PIC_ERR_INVALID_ARG;
   const long long n_sub = n_words / kQ;
   if (static_cast<long long>(workspace_bytes) < ws_size(n_sub, B, p)) return PIC_ERR_INVALID_ARG;
-  // 2 tables + the pass's words + the output staging rows + 2 pair tables
-  const size_t lut_smem = (sizeof(uint16_t) * 2 << p) + (kWbuf + kStageInts) * sizeof(uint32_t) + (2 << p);
-  int grid = 0;
-  int rc = decode_grid(p, lut_smem, &grid);
+    int grid = 0;
+  int rc = decode_grid(p, &grid);
   if (rc != PIC_OK) return rc;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   DecodeParams P{};
@@ -578,23 +729,28 @@ int pic_huffman_decode(const uint32_t* words, int64_t n_words, const int64_t* wo
   P.p = p;
   P.sym_off = reinterpret_cast<const long long*>(sym_off);
   P.tab_value = tab_value;
+  P.tab_len = tab_len;
   P.max_table = max_table;
   P.out = out;
   P.ws = ws_view(workspace, n_sub, B, p);
   P.n_sub = n_sub;
-  // whole passes of kThreads subsequences per CTA (no thread idles in a pass)
-  const long long passes = (n_sub + static_cast<long long>(grid) * kThreads - 1) /
-                           (static_cast<long long>(grid) * kThreads);
-  P.per_block = passes * kThreads;
-  if (cudaMemsetAsync(workspace, 0, 16 + kMaxPasses * 4, s) != cudaSuccess) {  // status, pass counters
-    cudaGetLastError();
-    return PIC_ERR_CUDA;
-  }
-  huff_lut<<<B, kThreads, 0, s>>>(tab_len, max_table, p, P.ws.lut, P.ws.status);
-  const long long g = (n_sub + P.per_block - 1) / P.per_block;
+  const long long groups = (n_sub + 31) / 32;
+  // the fewest rounds that the resident warps can do the groups in, and the
+  // warps per CTA that it takes
+  const long long rounds = (groups + kMaxWarps * grid - 1) / (kMaxWarps * grid);
+  const long long per = (groups + rounds * grid - 1) / (rounds * grid);
+  const int warps = static_cast<int>(per < kMinWarps ? kMinWarps : per);
+  // at least the CTAs that the tables can be made by: small images then have
+  // CTAs of their own, whose shared memory holds their tables (256 images of
+  // 64x64: 86 us packed, 38 us spread)
+  const long long g = std::min<long long>(std::max<long long>((groups + warps - 1) / warps, kMaxParts * (long long)B), grid);
+  P.groups_base = groups / g;
+  P.groups_more = static_cast<int>(groups % g);
+  P.parts = 1;
+  while (P.parts < kMaxParts && p >= 8 && 2LL * P.parts * B <= g) P.parts *= 2;
   void* args[] = {&P};
   if (cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(huff_decode), dim3(static_cast<unsigned>(g)),
-                                  dim3(kThreads), args, lut_smem, s) != cudaSuccess) {
+                                  dim3(32 * warps), args, smem_bytes(p, warps), s) != cudaSuccess) {
     cudaGetLastError();
     return PIC_ERR_CUDA;
   }
