@@ -2,12 +2,11 @@
 // behind the C ABI of include/pic_izpr.h.
 //
 // Algorithm 1 expands each block from its end-of-block marker offsets, which
-// the paper finds beforehand by a stream compaction.  Here:
-// 1. izpr_count: eob markers per 2048-symbol chunk (16-byte loads), summed
-//    over groups of 8 chunks, with each chunk's offset within its group.
-// 2. izpr_scan: one CTA, exclusive scan of the group counts; a chunk's
-//    first block = its group's base + its offset in the group.
-// 3. izpr_expand: persistent CTAs do the compaction and the expansion
+// the paper finds beforehand by a stream compaction.  Here, with the stream
+// cut into 2048-symbol chunks and the chunks into one contiguous range per CTA:
+// 1. izpr_count: the eob markers of each range.
+// 2. izpr_expand: each CTA adds up the ranges before its own, which is its
+//    first block, and does the compaction and the expansion of its chunks
 //    together, chunk by chunk, as a segmented scan.  Each thread holds 16
 //    consecutive symbols of the chunk in registers (loaded while the CTA
 //    expanded its previous chunk) and reduces them to (markers, positions
@@ -19,8 +18,15 @@
 //    the next zigzag position, a run code of n zeros skips n positions, a
 //    marker closes the block (its stream index is Algorithm 1's offset).  The
 //    blocks, assembled in shared memory, leave as whole 256-byte blocks.
-// The stream is read twice (steps 1 and 3); nothing else touches HBM but
-// the coefficients and offsets written.
+// The stream is read twice; nothing else touches HBM but the coefficients and
+// offsets written.
+//
+// What bounds it: small streams, the launches -- two; there were four (a
+// memset of the status word, and a scan by one CTA of counts that chunks dealt
+// out round robin needed) -- and large ones, the instructions of the walks (66 for 32 symbols).
+// Measured, before and now: one 768x512 image (407 k symbols) 16.7 -> 12.1 us,
+// the 64-image batch (26 M symbols) 100 -> 91.6 us, one symbol 15.2 -> 9.5 us.
+#include <algorithm>
 #include <cstdint>
 
 #include <cuda_runtime.h>
@@ -37,35 +43,28 @@ constexpr int kChunk = kThreads * kPerThread;  // symbols per compaction chunk
 
 enum : int { kBadBlock = 1, kBadCount = 2 };
 
-// Chunks are counted in groups of kGroup (one CTA of kGroup x kThreads
-// threads per group), so the scan runs over the groups.
-constexpr int kGroup = 8;
-// Workspace: status word, marker total, group counts, each chunk's first
-// block within its group, group bases.
+constexpr int kMaxGrid = 2048;  // ranges
+
+// Workspace: status word, and each range's markers.
 struct Workspace {
   int* status;
-  long long* total;
-  int* gcount;
-  int* local;
-  long long* gbase;
+  int* count;
 };
 __host__ __device__ inline long long n_chunks_of(long long n) { return (n + kChunk - 1) / kChunk; }
-__host__ __device__ inline long long n_groups_of(long long n) { return (n_chunks_of(n) + kGroup - 1) / kGroup; }
-__host__ __device__ inline long long align16(long long b) { return (b + 15) / 16 * 16; }
 __host__ __device__ inline long long ws_bytes(long long n) {
-  return 32 + align16(4 * n_groups_of(n)) + align16(4 * n_chunks_of(n)) + 8 * n_groups_of(n);
+  const long long c = n_chunks_of(n);
+  return 32 + ((c < kMaxGrid ? c : kMaxGrid) + 3) / 4 * 16;
 }
-__host__ __device__ inline Workspace ws_view(void* w, long long n) {
+__host__ __device__ inline Workspace ws_view(void* w) {
   char* p = static_cast<char*>(w);
-  const long long g = n_groups_of(n), c = n_chunks_of(n);
-  Workspace v;
-  v.status = reinterpret_cast<int*>(p);
-  v.total = reinterpret_cast<long long*>(p + 16);
-  v.gcount = reinterpret_cast<int*>(p + 32);
-  v.local = reinterpret_cast<int*>(p + 32 + align16(4 * g));
-  v.gbase = reinterpret_cast<long long*>(p + 32 + align16(4 * g) + align16(4 * c));
-  return v;
+  return Workspace{reinterpret_cast<int*>(p), reinterpret_cast<int*>(p + 32)};
 }
+// CTA i's chunks: `per` each, one more for the first `more` CTAs.
+struct Ranges {
+  long long per;
+  int more;
+  __device__ __forceinline__ long long first(int cta) const { return cta * per + min(cta, more); }
+};
 
 // Zigzag order of an 8x8 block (raster index of the k-th zigzag position):
 // anti-diagonal d = row + col, row falling for even d, rising for odd d.
@@ -106,105 +105,48 @@ __device__ __forceinline__ void load16(const int32_t* __restrict__ sym, long lon
   }
 }
 
-// Markers of the kGroup chunks of group blockIdx.x: thread t counts 16
-// symbols of chunk kGroup g + t / kThreads; the group's total, and each
-// chunk's count of markers before it within the group.
-__global__ void __launch_bounds__(kGroup * kThreads, 2) izpr_count(const int32_t* __restrict__ sym, long long n,
-                                                                int32_t eob, long long n_chunks, int* gcount,
-                                                                int* local) {
-  __shared__ int s_warp[kGroup * kThreads / 32];
-  const int t = threadIdx.x, sub = t / kThreads, lane = t & 31;
-  const long long c = static_cast<long long>(blockIdx.x) * kGroup + sub;
-  const long long i0 = c * kChunk + 16 * (t % kThreads);
+// The markers of each range.  What bounds it is DRAM, with 16-byte loads
+// coalesced over the CTA and kAhead of them in flight.
+constexpr int kCountThreads = 256;
+__global__ void __launch_bounds__(kCountThreads) izpr_count(const int32_t* __restrict__ sym, long long n, int32_t eob,
+                                                            Ranges ranges, Workspace ws) {
+  __shared__ int s_warp[kCountThreads / 32];
+  constexpr int kStep = 4 * kCountThreads, kAhead = 8;
+  const int t = threadIdx.x;
+  const bool vec = (reinterpret_cast<uintptr_t>(sym) & 15u) == 0;
+  const long long end = min(ranges.first(blockIdx.x + 1) * kChunk, n);
+  long long i = ranges.first(blockIdx.x) * kChunk + 4 * t;
   int cnt = 0;
-  if (c < n_chunks) {
-    int r[16];
-    load16(sym, n, i0, (reinterpret_cast<uintptr_t>(sym) & 15u) == 0, eob, r);
+  for (; vec && i + kStep * (kAhead - 1) + 3 < end; i += kStep * kAhead) {
+    int4 v[kAhead];
 #pragma unroll
-    for (int k = 0; k < 16; ++k) cnt += (r[k] == eob && i0 + k < n) ? 1 : 0;
+    for (int j = 0; j < kAhead; ++j) v[j] = __ldg(reinterpret_cast<const int4*>(sym + i) + kCountThreads * j);
+#pragma unroll
+    for (int j = 0; j < kAhead; ++j) cnt += (v[j].x == eob) + (v[j].y == eob) + (v[j].z == eob) + (v[j].w == eob);
   }
+  for (; i < end; i += kStep) {
+    if (vec && i + 3 < end) {
+      const int4 v = __ldg(reinterpret_cast<const int4*>(sym + i));
+      cnt += (v.x == eob) + (v.y == eob) + (v.z == eob) + (v.w == eob);
+    } else {
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
-  if (lane == 0) s_warp[t >> 5] = cnt;
+      for (int u = 0; u < 4; ++u) cnt += i + u < end && __ldg(sym + i + u) == eob;
+    }
+  }
+  cnt = __reduce_add_sync(0xffffffffu, cnt);
+  if (t % 32 == 0) s_warp[t / 32] = cnt;
   __syncthreads();
   if (t == 0) {
-    constexpr int kWarpsPerChunk = kThreads / 32;
-    int run = 0;
-    for (int q = 0; q < kGroup; ++q) {
-      const long long cq = static_cast<long long>(blockIdx.x) * kGroup + q;
-      if (cq < n_chunks) local[cq] = run;
-      for (int w = 0; w < kWarpsPerChunk; ++w) run += s_warp[q * kWarpsPerChunk + w];
-    }
-    gcount[blockIdx.x] = run;
+    for (int w = 1; w < kCountThreads / 32; ++w) cnt += s_warp[w];
+    ws.count[blockIdx.x] = cnt;
+    if (blockIdx.x == 0) *ws.status = 0;
   }
-}
-
-// One CTA: exclusive scan of the chunk counts into chunk bases; the total.
-// Tiles of 8192 counts are staged in shared memory by coalesced loads
-// (padded: entry j at j + j / 32); thread t scans entries 8t .. 8t+7.
-__global__ void __launch_bounds__(1024) izpr_scan(const int* __restrict__ counts, long long n_chunks,
-                                                  long long* base, long long* total) {
-  constexpr int kPer = 8, kTileN = 1024 * kPer;
-  __shared__ int s_c[kTileN + kTileN / 32];
-  __shared__ long long s_w[32];
-  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-  long long carry = 0;
-  for (long long t0 = 0; t0 < n_chunks; t0 += kTileN) {
-    const long long m = min(static_cast<long long>(kTileN), n_chunks - t0);
-    int v[kPer];  // all loads in flight together, then the shared stores
-#pragma unroll
-    for (int k = 0; k < kPer; ++k) {
-      const int j = t + 1024 * k;
-      v[k] = j < m ? __ldg(counts + t0 + j) : 0;
-    }
-#pragma unroll
-    for (int k = 0; k < kPer; ++k) {
-      const int j = t + 1024 * k;
-      s_c[j + (j >> 5)] = v[k];
-    }
-    __syncthreads();
-    long long s = 0;
-#pragma unroll
-    for (int k = 0; k < kPer; ++k) {
-      const int j = kPer * t + k;
-      s += s_c[j + (j >> 5)];
-    }
-    long long x = s;  // inclusive scan: warp, then warp totals
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const long long y = __shfl_up_sync(0xffffffffu, x, o);
-      if (lane >= o) x += y;
-    }
-    if (lane == 31) s_w[warp] = x;
-    __syncthreads();
-    if (warp == 0) {
-      long long w = s_w[lane];
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const long long y = __shfl_up_sync(0xffffffffu, w, o);
-        if (lane >= o) w += y;
-      }
-      s_w[lane] = w;
-    }
-    __syncthreads();
-    long long run = carry + (warp > 0 ? s_w[warp - 1] : 0) + x - s;
-#pragma unroll
-    for (int k = 0; k < kPer; ++k) {
-      const int j = kPer * t + k;
-      if (j < m) base[t0 + j] = run;
-      run += s_c[j + (j >> 5)];
-    }
-    carry += s_w[31];
-    __syncthreads();  // s_c and s_w are free again
-  }
-  if (t == 0) *total = carry;
 }
 
 // Compaction and expansion in one pass over the stream, as a segmented scan.
 // A block holds at most 64 symbols before its marker, so the marker that
 // precedes a chunk's first block lies within the kHalo symbols before the
-// chunk (or the block is malformed).  Persistent CTAs take chunks c,
-// c + grid, ...; for each:
+// chunk (or the block is malformed).  For each chunk of the CTA's range:
 //  - every thread holds 16 consecutive symbols of the chunk in registers
 //    (loaded while the CTA worked on its previous chunk) and reduces them to
 //    (markers, positions covered since its last marker);
@@ -212,7 +154,7 @@ __global__ void __launch_bounds__(1024) izpr_scan(const int* __restrict__ counts
 //    the chunk's first block that lies in the halo (they carry in);
 //  - a CTA-wide segmented scan of the (markers, positions) pairs gives each
 //    thread the block of its first symbol (block q of the chunk = block
-//    base[chunk] + q of the stream) and the zigzag position reached in it;
+//    gb0 + q of the stream) and the zigzag position reached in it;
 //  - each thread walks its symbols: a literal goes to the block's next
 //    zigzag position, a run code of n zeros skips n positions, a marker
 //    closes the block (its stream index is Algorithm 1's offset);
@@ -240,9 +182,8 @@ __device__ __forceinline__ Seg seg_cat(Seg a, Seg b) { return Seg{a.m + b.m, b.m
 
 __global__ void __launch_bounds__(kThreads, 8) izpr_expand(const int32_t* __restrict__ sym,
                                                         long long n, int32_t eob,
-                                                        const long long* __restrict__ gbase,
-                                                        const int* __restrict__ local,
-                                                        const long long* total, long long n_blocks,
+                                                        Ranges ranges, const int* __restrict__ count,
+                                                        long long n_blocks,
                                                         int32_t* __restrict__ coeffs,
                                                         int64_t* __restrict__ offsets, int* status) {
   extern __shared__ __align__(16) unsigned char smem[];
@@ -252,10 +193,9 @@ __global__ void __launch_bounds__(kThreads, 8) izpr_expand(const int32_t* __rest
   int* s_carry = reinterpret_cast<int*>(s_zz + 64);
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
   constexpr int kWarps = kThreads / 32;
-  const long long n_chunks = (n + kChunk - 1) / kChunk;
+  const long long c_begin = ranges.first(blockIdx.x), c_end = ranges.first(blockIdx.x + 1);
   if (t < 64) s_zz[t] = static_cast<unsigned char>(make_zigzag().v[t]);
   if (blockIdx.x == 0 && t == 0) {
-    if (*total != n_blocks) atomicOr(status, kBadCount);
     if (__ldg(sym + n - 1) != eob) atomicOr(status, kBadCount);  // symbols after the last marker
   }
   for (int j = t; j < (kMaxBlk + 1) * kBlkStride / 4; j += kThreads)
@@ -274,26 +214,49 @@ __global__ void __launch_bounds__(kThreads, 8) izpr_expand(const int32_t* __rest
     for (int u = 0; u < 3; ++u) h[u] = (warp != 0 || hi + u < 0) ? eob : __ldg(sym + hi + u);
   };
 
-  // the next chunk's symbols, halo and first block index, loaded one chunk ahead
+  // the next chunk's symbols and halo, loaded one chunk ahead
   int cur[16], hcur[3];
-  long long bcur = 0;
-  if (blockIdx.x < n_chunks) {
-    load16(sym, n, static_cast<long long>(blockIdx.x) * kChunk + 16 * t, vec, fill, cur);
-    load_halo(blockIdx.x, hcur);
-    bcur = gbase[blockIdx.x / kGroup] + local[blockIdx.x];
+  load16(sym, n, c_begin * kChunk + 16 * t, vec, fill, cur);
+  load_halo(c_begin, hcur);
+  // the blocks of the ranges before this one; of all ranges
+  long long gb0 = 0;
+  {
+    long long before = 0, all = 0;
+    for (int i = t; i < static_cast<int>(gridDim.x); i += kThreads) {
+      const int v = count[i];
+      before += i < static_cast<int>(blockIdx.x) ? v : 0;
+      all += v;
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      before += __shfl_xor_sync(0xffffffffu, before, o);
+      all += __shfl_xor_sync(0xffffffffu, all, o);
+    }
+    long long* s_sum = reinterpret_cast<long long*>(s_scan);
+    if (lane == 0) {
+      s_sum[2 * warp] = before;
+      s_sum[2 * warp + 1] = all;
+    }
+    __syncthreads();
+    all = 0;
+#pragma unroll
+    for (int w = 0; w < kWarps; ++w) {
+      gb0 += s_sum[2 * w];
+      all += s_sum[2 * w + 1];
+    }
+    if (blockIdx.x == 0 && t == 0 && all != n_blocks) atomicOr(status, kBadCount);
+    __syncthreads();
   }
-  for (long long c = blockIdx.x; c < n_chunks; c += gridDim.x) {
+  for (long long c = c_begin; c < c_end; ++c) {
     const long long c0 = c * kChunk;
-    const long long gb0 = bcur;
     int x16[16], h[3];
 #pragma unroll
     for (int i = 0; i < 16; ++i) x16[i] = cur[i];
 #pragma unroll
     for (int u = 0; u < 3; ++u) h[u] = hcur[u];
-    if (c + gridDim.x < n_chunks) {  // next chunk, in flight meanwhile
-      load16(sym, n, (c + gridDim.x) * kChunk + 16 * t, vec, fill, cur);
-      load_halo(c + gridDim.x, hcur);
-      bcur = gbase[(c + gridDim.x) / kGroup] + local[c + gridDim.x];
+    if (c + 1 < c_end) {  // next chunk, in flight meanwhile
+      load16(sym, n, (c + 1) * kChunk + 16 * t, vec, fill, cur);
+      load_halo(c + 1, hcur);
     }
 
     // this thread's markers (bit i: symbol i) and positions since its last one
@@ -418,16 +381,16 @@ __global__ void __launch_bounds__(kThreads, 8) izpr_expand(const int32_t* __rest
       __syncthreads();  // the slots are clear again
     }
     if (bad) atomicOr(status, kBadBlock);
+    gb0 += tot;
     __syncthreads();  // the scan scratch and the halo carry are free again
   }
 }
 
-__global__ void izpr_flag(int* status, int bits) { atomicOr(status, bits); }
+__global__ void izpr_flag(int* status, int bits) { *status = bits; }
 
 bool aligned(const void* p, uintptr_t a) { return (reinterpret_cast<uintptr_t>(p) % a) == 0; }
 
-// Persistent grid of izpr_expand on the current device (resident CTAs over
-// all SMs), set up once per device.
+// Resident CTAs of izpr_expand on the current device, set up once per device.
 int expand_grid(int* grid) {
   constexpr int kMaxDev = 64;
   static int cached[kMaxDev];
@@ -447,7 +410,7 @@ int expand_grid(int* grid) {
       cudaGetLastError();
       return PIC_ERR_CUDA;
     }
-    cached[dev] = sms * per_sm;
+    cached[dev] = std::min(sms * per_sm, kMaxGrid);
   }
   *grid = cached[dev];
   return PIC_OK;
@@ -475,23 +438,18 @@ int pic_izpr_decode(const int32_t* symbols, int64_t n_symbols, int32_t eob, int6
     return PIC_ERR_INVALID_ARG;
   if (eob < INT32_MIN + 17) return PIC_ERR_INVALID_ARG;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  Workspace ws = ws_view(workspace, n_symbols);
+  const Workspace ws = ws_view(workspace);
   const long long chunks = n_chunks_of(n_symbols);
-  if (cudaMemsetAsync(workspace, 0, 32, s) != cudaSuccess) {  // status and total start at zero
-    cudaGetLastError();
-    return PIC_ERR_CUDA;
-  }
   if (chunks > 0) {
-    const long long groups = n_groups_of(n_symbols);
-    izpr_count<<<static_cast<unsigned>(groups), kGroup * kThreads, 0, s>>>(symbols, n_symbols, eob, chunks,
-                                                                           ws.gcount, ws.local);
-    izpr_scan<<<1, 1024, 0, s>>>(ws.gcount, groups, ws.gbase, ws.total);
     int grid = 0;
     if (expand_grid(&grid) != PIC_OK) return PIC_ERR_CUDA;
-    izpr_expand<<<static_cast<unsigned>(chunks < grid ? chunks : grid), kThreads, kExpandSmem, s>>>(
-        symbols, n_symbols, eob, ws.gbase, ws.local, ws.total, n_blocks, coeffs, offsets, ws.status);
-  } else if (n_blocks > 0) {
-    izpr_flag<<<1, 1, 0, s>>>(ws.status, kBadCount);  // no symbols, hence no markers
+    const int g = static_cast<int>(std::min<long long>(chunks, grid));
+    const Ranges ranges{chunks / g, static_cast<int>(chunks % g)};
+    izpr_count<<<g, kCountThreads, 0, s>>>(symbols, n_symbols, eob, ranges, ws);
+    izpr_expand<<<g, kThreads, kExpandSmem, s>>>(symbols, n_symbols, eob, ranges, ws.count, n_blocks, coeffs, offsets,
+                                                 ws.status);
+  } else {
+    izpr_flag<<<1, 1, 0, s>>>(ws.status, n_blocks > 0 ? kBadCount : 0);  // no symbols, hence no markers
   }
   if (cudaGetLastError() != cudaSuccess) return PIC_ERR_CUDA;
   return PIC_OK;
