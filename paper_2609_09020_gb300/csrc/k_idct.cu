@@ -13,17 +13,21 @@
 //           (a warp reads 4 whole patches, 1 KB contiguous) one pass ahead,
 //           scales them by the level's step and stores them into the
 //           patch's shared slot;
-//   pass 1  thread j transforms column j: T[m][j] = sum_u c[u][m] S[u][j];
-//   pass 2  thread j transforms row j:    x[j][n] = sum_v c[v][n] T[j][v];
-//   store   lanes 2i and 2i+1 trade row halves so that each store
-//           instruction writes whole 32-byte rows: row 2i in the first,
-//           row 2i+1 in the second.
+//   pass 1  thread j transforms row j:    T[j][n] = sum_v c[v][n] S[j][v];
+//   pass 2  thread j transforms column j: x[m][j] = sum_u c[u][m] T[u][j];
+//   store   thread j holds column j, so a warp stores, row by row, 32
+//           consecutive floats of a latent row: whole lines at any alignment.
+//           (With the columns first, thread j held a row, and rows of odd
+//           width went out as four-byte pieces of eight rows at a time.)
+// Measured, before and now: 12 photos of 683x1021, two channels, 43.6 -> 39.5
+// us (178 MB; 26.4 us at the copy rate), 12 of 688x1024 35.9 both.  More CTAs
+// or coefficients in flight, or a CTA per pass, give nothing: 35 to 39 us.
 // Each 1-D transform x[n] = sum_k a(k) X[k] cos((2n + 1) k pi / 16) is the
 // even/odd split of the basis (cos((2(7-n) + 1) k pi / 16) = (-1)^k times
 // that of n): x[n] = E[n] + O[n], x[7-n] = E[n] - O[n] with E the 4-point
 // transform of X[0, 2, 4, 6] (split once more) and O a 4x4 product of
 // X[1, 3, 5, 7] -- 36 operations instead of 64 multiply-adds.  The patch
-// slot is padded to 72 floats so the column accesses of pass 1 hit 32
+// slot is padded to 72 floats so the column accesses of pass 2 hit 32
 // distinct banks.
 #include <cstdint>
 
@@ -103,7 +107,6 @@ __global__ void __launch_bounds__(kThreads, 6)
   const int t = threadIdx.x;
   const int slot = t >> 3;
   const int j = t & 7;
-  const int odd = j & 1;
   float* my = tile + slot * kSlot;
 
   const int stride = static_cast<int>(gridDim.x) * kPatches;
@@ -144,58 +147,32 @@ __global__ void __launch_bounds__(kThreads, 6)
     v1 = n1;
     __syncwarp();
 
-    // pass 1: column j, vertical inverse transform
-    float col[8], tr[8];
-#pragma unroll
-    for (int u = 0; u < 8; ++u) col[u] = my[u * 8 + j];
-    idct8(col, tr);
-    __syncwarp();
-#pragma unroll
-    for (int m = 0; m < 8; ++m) my[m * 8 + j] = tr[m];
-    __syncwarp();
-
-    // pass 2: row j, horizontal inverse transform
+    // pass 1: row j, horizontal inverse transform
     const float4 r0 = reinterpret_cast<const float4*>(my)[2 * j];
     const float4 r1 = reinterpret_cast<const float4*>(my)[2 * j + 1];
     const float row[8] = {r0.x, r0.y, r0.z, r0.w, r1.x, r1.y, r1.z, r1.w};
-    float x[8];
-    idct8(row, x);
+    float tr[8], col[8], x[8];
+    idct8(row, tr);
+    __syncwarp();
+    reinterpret_cast<float4*>(my)[2 * j] = make_float4(tr[0], tr[1], tr[2], tr[3]);
+    reinterpret_cast<float4*>(my)[2 * j + 1] = make_float4(tr[4], tr[5], tr[6], tr[7]);
+    __syncwarp();
+
+    // pass 2: column j, vertical inverse transform
+#pragma unroll
+    for (int u = 0; u < 8; ++u) col[u] = my[u * 8 + j];
+    idct8(col, x);
     __syncwarp();  // the slot is refilled by the next pass
 
-    // lanes 2i, 2i+1: the even lane sends its right half, the odd lane its left
-    float recv[4];
-#pragma unroll
-    for (int n = 0; n < 4; ++n) recv[n] = __shfl_xor_sync(0xffffffffu, odd ? x[n] : x[4 + n], 1);
-    // store 0 writes row j & ~1 (even lane: columns 0-3 of its own row; odd
-    // lane: columns 4-7 received), store 1 row j | 1 (even lane: columns 0-3
-    // received; odd lane: columns 4-7 of its own row)
-    const float4 s0 = odd ? make_float4(recv[0], recv[1], recv[2], recv[3])
-                          : make_float4(x[0], x[1], x[2], x[3]);
-    const float4 s1 = odd ? make_float4(x[4], x[5], x[6], x[7])
-                          : make_float4(recv[0], recv[1], recv[2], recv[3]);
     if (live) {
       const Plane& P = p.pl[pi];
       const int pr = k - P.blk0;
       const int by = static_cast<int>(udiv(pr, P.bw, P.bw_inv)), bx = pr - by * P.bw;
-      const int q0 = 8 * bx + 4 * odd;
-      const int nv = min(4, P.Wl - q0);  // valid columns of this half (may be <= 0)
-      float* plane = p.latents + b * p.lat_per_image + P.lat_off + q0;
+      const int rows = 8 * bx + j < P.Wl ? P.Hl - 8 * by : 0;  // valid ones of this column
+      float* dst = p.latents + b * p.lat_per_image + P.lat_off + static_cast<long long>(8 * by) * P.Wl + 8 * bx + j;
 #pragma unroll
-      for (int e = 0; e < 2; ++e) {
-        const int r = 8 * by + (e ? (j | 1) : (j & ~1));
-        const float4 sv = e ? s1 : s0;
-        if (r < P.Hl && nv > 0) {
-          float* dst = plane + static_cast<long long>(r) * P.Wl;
-          if (nv == 4 && (reinterpret_cast<uintptr_t>(dst) & 15u) == 0) {
-            *reinterpret_cast<float4*>(dst) = sv;
-          } else {
-            const float vv[4] = {sv.x, sv.y, sv.z, sv.w};
-#pragma unroll
-            for (int n = 0; n < 4; ++n)
-              if (n < nv) dst[n] = vv[n];
-          }
-        }
-      }
+      for (int m = 0; m < 8; ++m)
+        if (m < rows) dst[static_cast<long long>(m) * P.Wl] = x[m];
     }
   }
 }
@@ -203,6 +180,28 @@ __global__ void __launch_bounds__(kThreads, 6)
 bool sizes_ok(int H, int W, int L, int C) {
   return H >= 1 && W >= 1 && H <= 65536 && W <= 65536 && L >= 1 && L <= kLevelsMax && C >= 1 &&
          C <= kChanMax;
+}
+
+// Resident CTAs of the kernel on the current device, set up once per device.
+int idct_grid(int* grid) {
+  constexpr int kMaxDev = 64;
+  static int cached[kMaxDev];
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDev) {
+    cudaGetLastError();
+    return PIC_ERR_CUDA;
+  }
+  if (cached[dev] == 0) {
+    int sms = 0, per_sm = 0;
+    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, idct_unpatchify_kernel, kThreads, 0) != cudaSuccess) {
+      cudaGetLastError();
+      return PIC_ERR_CUDA;
+    }
+    cached[dev] = sms * (per_sm > 0 ? per_sm : 1);
+  }
+  *grid = cached[dev];
+  return PIC_OK;
 }
 
 }  // namespace
@@ -252,16 +251,9 @@ extern "C" int pic_idct_unpatchify(const int32_t* coeffs, const float* steps, in
   p.lat_per_image = off;
   p.total_blocks = static_cast<int>(blk * B);
 
-  int dev = 0, sms = 0, per_sm = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess ||
-      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, idct_unpatchify_kernel, kThreads, 0) !=
-          cudaSuccess) {
-    cudaGetLastError();
-    return PIC_ERR_CUDA;
-  }
+  int cap = 0;
+  if (idct_grid(&cap) != PIC_OK) return PIC_ERR_CUDA;
   const long long passes = (p.total_blocks + kPatches - 1) / kPatches;
-  const long long cap = static_cast<long long>(sms) * (per_sm > 0 ? per_sm : 1);
   const unsigned grid = static_cast<unsigned>(passes < cap ? passes : cap);
   idct_unpatchify_kernel<<<grid, kThreads, 0, static_cast<cudaStream_t>(stream)>>>(p);
   if (cudaGetLastError() != cudaSuccess) return PIC_ERR_CUDA;
