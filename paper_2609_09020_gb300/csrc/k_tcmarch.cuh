@@ -33,7 +33,8 @@
 // a cycle).  64 images of 768x512: 705 us with the per-tile kernel, whose
 // decoding warps also staged and interpolated the features, 660 us here;
 // 14-64-64-3 at 1361x2041, two images: 228 -> 183 us; 16-64-64-64-3 GELU at
-// 3840x2160, whose FP32 pipe is bound by the GELUs: 1020 -> 990 us.
+// 3840x2160, bound by the GELUs: 1020 -> 990 us (836 with the GELU of
+// pic_common.cuh as it is now).
 // Both thin layers, or the output layer alone, by warp-level mma.sync on
 // accumulator fragments (one round trip less) measured 740 and 779 us:
 // mma.sync shares the tensor pipe with tcgen05, waits whenever that is busy,

@@ -1,37 +1,25 @@
 // Generated by paper_2609_09020_gb300/gen_gelu.py -- do not edit.
-// Phi(z) - 1/2 ~= z * P(s) / Q(s), s = min(z^2, 5.1^2); max |GELU error|
-// in fp32 ~ 1.2e-06.
+// Phi(-a) ~= 2^q(-a) on 0 <= a <= 5.8; max |GELU error| in fp32 ~ 5.2e-07.
 #pragma once
 
 namespace pic {
 
-constexpr float kGeluZ2 = 26.010000228881836f;  // Z^2
-constexpr int kGeluDegP = 5;
-constexpr int kGeluDegQ = 4;
+constexpr float kGeluZ = 5.800000190734863f;
+constexpr float kGeluEps = 3.301103168595887e-09f;  // just above 2^q(-Z)
+constexpr int kGeluDeg = 6;
 
-// Coefficients of P and Q, highest degree first (Horner order); Q's last is 1.
-__host__ __device__ constexpr float gelu_p(int i) {
+// Coefficients of q, highest degree first (Horner order).
+__host__ __device__ constexpr float gelu_c(int i) {
   constexpr float c[] = {
-      -1.9798260808556734e-08f,
-      6.712000867992174e-06f,
-      0.0005090613849461079f,
-      0.006648619659245014f,
-      0.06904540956020355f,
-      0.3989395797252655f,
-  };
-  return c[i];
-}
-
-__host__ __device__ constexpr float gelu_q(int i) {
-  constexpr float c[] = {
-      0.00017359455523546785f,
-      0.0037839559372514486f,
-      0.048325538635253906f,
-      0.3397088646888733f,
-      1.0f,
+      3.3092816011048853e-05f,
+      0.0007692197104915977f,
+      0.008080716244876385f,
+      0.05341210216283798f,
+      -0.4587709605693817f,
+      1.1512017250061035f,
+      -0.999993085861206f,
   };
   return c[i];
 }
 
 }  // namespace pic
-

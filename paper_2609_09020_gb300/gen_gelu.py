@@ -1,130 +1,107 @@
-"""Generates the rational function behind the CUDA path's GELU
-(csrc/pic_gelu.cuh).
+"""Generates the polynomial behind the CUDA path's GELU (csrc/pic_gelu.cuh).
 
-GELU(z) = z Phi(z), Phi(z) = (1 + erf(z / sqrt 2)) / 2.  On |z| <= Z, Z = 5.1,
+GELU(z) = z Phi(z), Phi(z) = (1 + erf(z / sqrt 2)) / 2.  With a = |z|,
 
-    Phi(z) - 1/2 ~= z * R(s),   R(s) = P(s) / Q(s),   s = min(z^2, Z^2),
+    GELU(z) = max(z, 0) - a Phi(-a),   Phi(-a) ~= 2^q(a),
 
-P of degree 5 and Q of degree 4 with Q(0) = 1 and Q >= 1 on [0, Z^2] (so the
-reciprocal is well conditioned).  Phi = saturate(1/2 + z R(s)): the
-saturation clamps Phi to [0, 1] and handles |z| > Z, where Phi(-Z) = 1.7e-7.
-The GELU error is z (z R - (Phi(z) - 1/2)), so R is fitted to
-(Phi(z) - 1/2) / z with weight z^2: the rational least-squares problem is
-linearised as P(s) - f Q(s) ~= 0 and re-solved with weights 1 / |Q| from the
-previous pass (Loeb's iteration), while Lawson's reweighting raises the
-weight of the points where the error is largest, turning the fit into a
-minimax one; the fit runs in the scaled variable s / Z^2 on Chebyshev nodes
-of [0, Z] and the coefficients are then rescaled for s itself.  The kernels
-evaluate P and Q by Horner's rule (9 multiply-adds), one reciprocal
-(rcp.approx, on the special-function unit) and four more operations:
-z^2, P * (1 / Q), the saturating multiply-add and z Phi.  Against the
-degree-12 polynomial in the same variable this takes 13 instead of 16
-FP32-pipe operations per value at the same accuracy.  The maximum GELU
-error over the real line with the fp32 evaluation order of the kernels
-(measured below on a grid of 1.2 M points of [-12, 12], the reciprocal
-correctly rounded) is printed into the header.
+q of degree 6 on 0 <= a <= Z, Z = 5.8: log2 Phi(-a) is close to a parabola,
+so a low degree does.  Beyond Z the subtracted part, below 2e-8, is to vanish
+exactly: a is clamped at Z, and the kernels subtract EPS, a little more than
+2^q(Z), from the power and clamp the difference at zero.  An error d in q
+is an error a Phi(-a) ln 2 d of the GELU, so q is fitted to log2 Phi(-a)
+with that weight; Lawson's reweighting raises the weight of the points where
+the error is largest, turning the least-squares fit into a minimax one.  It
+runs in the scaled variable a / Z on Chebyshev nodes of [0, Z]; the
+coefficients are then rescaled for -a, the variable that the kernels keep
+(so that the last step is a multiply-add).  Per value the kernels take two
+minima or maxima, 6 multiply-adds by Horner's rule, one 2^x (ex2.approx, on
+the special-function unit), a saturating subtraction and the last
+multiply-add.  The maximum GELU error over the real line with the fp32
+evaluation order of the kernels (measured below on a grid of 1.2 M points of
+[-12, 12], the power correctly rounded) is printed into the header; most of
+it is the rounding of the result itself.
 
 Run:  python -m paper_2609_09020_gb300.gen_gelu  (prints the header)
 """
 from __future__ import annotations
 
 import numpy as np
-from scipy.special import erf
+from scipy.special import erf, erfc
 
-Z = 5.1
-DEG_P = 5
-DEG_Q = 4
-PASSES = 80
+Z = 5.8
+DEG = 6
+PASSES = 200
 
 
 def fit():
-    """Coefficients (p, q) of P and Q in s = min(z^2, Z^2), lowest degree
-    first, q[0] = 1."""
+    """Coefficients of q as a polynomial in -a, lowest degree first, and EPS."""
     n = 12000
-    zs = 0.5 * Z * (1 - np.cos(np.pi * (np.arange(n) + 0.5) / n))
-    zs = np.concatenate([zs, np.linspace(1e-4, Z, n)])
-    x = zs ** 2 / Z ** 2                     # scaled variable in [0, 1]
-    f = 0.5 * erf(zs / np.sqrt(2)) / zs      # (Phi(z) - 1/2) / z
-    w = zs ** 2                              # GELU error = z^2 (R - f)
-    vp = x[:, None] ** np.arange(DEG_P + 1)
-    vq = x[:, None] ** np.arange(1, DEG_Q + 1)
-    lw = np.ones_like(zs)
-    q_val = np.ones_like(zs)
+    a = 0.5 * Z * (1 - np.cos(np.pi * (np.arange(n) + 0.5) / n))
+    phi = 0.5 * erfc(a / np.sqrt(2))
+    f = np.log2(phi)
+    w = a * phi * np.log(2)
+    v = (a[:, None] / Z) ** np.arange(DEG + 1)
+    lw = np.ones_like(a)
     best = None
     for _ in range(PASSES):
-        a = np.concatenate([vp, -f[:, None] * vq], 1)
-        wt = w * lw / np.abs(q_val)
-        c, *_ = np.linalg.lstsq(a * wt[:, None], f * wt, rcond=None)
-        p, q = c[:DEG_P + 1], np.concatenate([[1.0], c[DEG_P + 1:]])
-        q_val = vq @ q[1:] + 1.0
-        e = np.abs((vp @ p / q_val - f) * w)
+        wt = w * lw
+        c, *_ = np.linalg.lstsq(v * wt[:, None], f * wt, rcond=None)
+        e = np.abs((v @ c - f) * w)
         if best is None or e.max() < best[0]:
-            best = (e.max(), p.copy(), q.copy())
+            best = (e.max(), c.copy())
         lw *= np.sqrt(e / e.max() + 1e-3)
         lw /= lw.max()
-    _, p, q = best
-    scale = (1.0 / Z ** 2) ** np.arange(max(DEG_P, DEG_Q) + 1)
-    return p * scale[:DEG_P + 1], q * scale[:DEG_Q + 1]
+    c = best[1] * (-1.0 / Z) ** np.arange(DEG + 1)
+    return c, float(2.0 ** np.polyval(c[::-1], -Z) * (1 + 1e-3))
 
 
 def _fma32(a, b, c):
     """fp32 fused multiply-add: the product of two fp32 values is exact in
     fp64, so one rounding of the fp64 sum to fp32 stands in for the FMA's."""
-    return (a.astype(np.float64) * b + np.float64(c)).astype(np.float32)
+    return (a.astype(np.float64) * b + np.asarray(c, np.float64)).astype(np.float32)
 
 
-def gelu_fp32(z: np.ndarray, pq) -> np.ndarray:
+def gelu_fp32(z: np.ndarray, coeffs) -> np.ndarray:
     """fp32 emulation of the CUDA evaluation order (the scalar and the pair
     form round identically: every step is one correctly rounded fp32
-    operation; the reciprocal is taken correctly rounded here, within an
-    ulp of the kernels' rcp.approx)."""
-    p, q = pq
+    operation; the power is taken correctly rounded here, within two ulps of
+    the kernels' ex2.approx)."""
+    c, eps = coeffs
     f32 = np.float32
     z = z.astype(f32)
-    s = np.minimum((z * z).astype(f32), f32(Z * Z))
-    pn = np.full_like(z, f32(p[-1]))
-    for a in p[-2::-1]:
-        pn = _fma32(pn, s, float(f32(a)))
-    qd = np.full_like(z, f32(q[-1]))
-    for a in q[-2::-1]:
-        qd = _fma32(qd, s, float(f32(a)))
-    r = (np.float64(1.0) / qd.astype(np.float64)).astype(f32)
-    rr = (pn * r).astype(f32)
-    phi = np.clip(_fma32(z, rr, 0.5), 0, 1).astype(f32)
-    return (z * phi).astype(f32)
+    na = np.maximum(-np.abs(z), f32(-Z))
+    q = np.full_like(z, f32(c[-1]))
+    for k in c[-2::-1]:
+        q = _fma32(q, na, float(f32(k)))
+    e = np.exp2(q.astype(np.float64)).astype(f32)
+    e = np.clip((e - f32(eps)).astype(f32), 0, 1)
+    return _fma32(na, e.astype(np.float64), np.maximum(z, f32(0)))
 
 
-def min_denominator(pq) -> float:
-    """Smallest Q(s) over s in [0, Z^2] (fp64)."""
-    _, q = pq
-    s = np.linspace(0.0, Z * Z, 100001)
-    return float(np.min(np.polyval(q[::-1], s)))
+def min_denominator(coeffs) -> float:
+    """The smallest value that the evaluation divides by: it has no division."""
+    return 1.0
 
 
-def max_error(pq) -> float:
+def max_error(coeffs) -> float:
     z = np.linspace(-12, 12, 1_200_001)
     ref = 0.5 * z * (1 + erf(z / np.sqrt(2)))
-    return float(np.max(np.abs(gelu_fp32(z, pq).astype(np.float64) - ref)))
+    return float(np.max(np.abs(gelu_fp32(z, coeffs).astype(np.float64) - ref)))
 
 
-def header(pq) -> str:
-    p, q = pq
+def header(coeffs) -> str:
+    c, eps = coeffs
     lines = ["// Generated by paper_2609_09020_gb300/gen_gelu.py -- do not edit.",
-             f"// Phi(z) - 1/2 ~= z * P(s) / Q(s), s = min(z^2, {Z}^2); max |GELU error|",
-             f"// in fp32 ~ {max_error(pq):.1e}.",
+             f"// Phi(-a) ~= 2^q(-a) on 0 <= a <= {Z}; max |GELU error| in fp32 ~ {max_error(coeffs):.1e}.",
              "#pragma once", "", "namespace pic {", "",
-             f"constexpr float kGeluZ2 = {float(np.float32(Z * Z))!r}f;  // Z^2",
-             f"constexpr int kGeluDegP = {DEG_P};",
-             f"constexpr int kGeluDegQ = {DEG_Q};",
+             f"constexpr float kGeluZ = {float(np.float32(Z))!r}f;",
+             f"constexpr float kGeluEps = {float(np.float32(eps))!r}f;  // just above 2^q(-Z)",
+             f"constexpr int kGeluDeg = {DEG};",
              "",
-             "// Coefficients of P and Q, highest degree first (Horner order); Q's last is 1.",
-             "__host__ __device__ constexpr float gelu_p(int i) {",
+             "// Coefficients of q, highest degree first (Horner order).",
+             "__host__ __device__ constexpr float gelu_c(int i) {",
              "  constexpr float c[] = {"]
-    lines += [f"      {float(np.float32(a))!r}f," for a in p[::-1]]
-    lines += ["  };", "  return c[i];", "}", "",
-              "__host__ __device__ constexpr float gelu_q(int i) {",
-              "  constexpr float c[] = {"]
-    lines += [f"      {float(np.float32(a))!r}f," for a in q[::-1]]
+    lines += [f"      {float(np.float32(k))!r}f," for k in c[::-1]]
     lines += ["  };", "  return c[i];", "}", "", "}  // namespace pic", ""]
     return "\n".join(lines)
 
