@@ -32,9 +32,9 @@
 // batches) and the issue slots (680 warp instructions a tile and warp, 0.68
 // a cycle).  64 images of 768x512: 705 us with the per-tile kernel, whose
 // decoding warps also staged and interpolated the features, 660 us here;
-// 14-64-64-3 at 1361x2041, two images: 228 -> 183 us; 16-64-64-64-3 GELU at
-// 3840x2160, bound by the GELUs: 1020 -> 990 us (836 with the GELU of
-// pic_common.cuh as it is now).
+// 14-64-64-3 at 1361x2041, two images: 228 -> 174 us; 16-64-64-64-3 GELU at
+// 3840x2160, bound by the GELUs: 1020 -> 990 us (789 with the GELU of
+// pic_common.cuh and the operands in two parts).
 // Both thin layers, or the output layer alone, by warp-level mma.sync on
 // accumulator fragments (one round trip less) measured 740 and 779 us:
 // mma.sync shares the tensor pipe with tcgen05, waits whenever that is busy,
@@ -60,6 +60,13 @@ struct MarchNet {
   static constexpr int L = L_, C = C_, NL = NL_, N = 64, ACT = ACT_;
   using F = FeatLayout<L, C>;
   static constexpr int K1 = F::K1, HID = NL - 2;
+  // An operand is handed to the tensor pipe in two parts, its first 16 columns
+  // ahead of the rest: the MMAs of the first part, and the better part of
+  // their round trip, run beside the rest of the epilogue.  16-64-64-64-3 GELU
+  // at 3840x2160: 836 us in one part, 789 cut after 16 columns, 825 after 32,
+  // 890 after 48; 7-64-64-3, one 768x512 image 20.4 -> 19.1 us, 64 of them
+  // the same; 14-64-64-3, one image of 1361x2041 70.0 -> 67.5 us.
+  static constexpr int CUT = 1;
   static constexpr int THREADS = 32 * (kDecWarps + kFeatWarps + kGroups);
   // 896 threads x 72 registers at launch, moved between the roles'
   // warpgroups (within the launch's total; below 96 the feature warps spill,
@@ -147,8 +154,8 @@ __device__ __forceinline__ bool wait_phase(uint32_t bar, uint32_t parity, volati
 
 // One pixel's accumulator row in region t -> activation, hi/lo split -> the
 // next layer's operand in place (per 16 columns: 8 of hi pairs, 8 of lo).
-template <class Net>
-__device__ __forceinline__ void epilogue(uint32_t t) {
+template <class Net, class Part>
+__device__ __forceinline__ void epilogue(uint32_t t, Part part_done) {
   uint32_t acc[2][16];
   tc::tmem_ld16(t, acc[0]);
 #pragma unroll
@@ -160,8 +167,11 @@ __device__ __forceinline__ void epilogue(uint32_t t) {
     for (int q = 0; q < 8; ++q)
       act_split<Net::ACT>(__uint_as_float(acc[c & 1][2 * q]), __uint_as_float(acc[c & 1][2 * q + 1]), hl[q], hl[8 + q]);
     tc::tmem_st16(t + 16 * c, hl);
+    if (c + 1 == Net::CUT || c + 1 == Net::N / 16) {
+      tc::tmem_st_wait();
+      part_done(c + 1 == Net::CUT);
+    }
   }
-  tc::tmem_st_wait();
 }
 
 template <class Net, bool FL>
@@ -175,13 +185,16 @@ __global__ void __launch_bounds__(Net::THREADS) __maxnreg__(Net::MAXREG)
   const uint32_t sbase = smem_addr(smem);
   // mbarriers, 8 bytes each, per group: feat_full (layer 0's operand written;
   // one arrival per feature warp), feat_free (read), acc0_full (layer 0
-  // done), acc_full (another layer done), a_full (a hidden operand written;
-  // one arrival per decoding warp), drain (the issuing warp's end).
+  // done), acc_full (another layer done), a_full and a2_full (the first and
+  // second part of a hidden operand written; one arrival per decoding warp;
+  // two barriers, since a warp may finish both parts before the issuing warp
+  // looks for the first), drain (the issuing warp's end).
   const uint32_t bar_ff = sbase, bar_fe = sbase + 8 * kGroups, bar_c0 = sbase + 16 * kGroups,
-                 bar_c = sbase + 24 * kGroups, bar_a = sbase + 32 * kGroups, bar_drain = sbase + 40 * kGroups;
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + 48 * kGroups);
+                 bar_c = sbase + 24 * kGroups, bar_a = sbase + 32 * kGroups, bar_a2 = sbase + 40 * kGroups,
+                 bar_drain = sbase + 48 * kGroups;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + 56 * kGroups);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 2);
-  static_assert(48 * kGroups + 16 <= Net::CTRL, "control block");
+  static_assert(56 * kGroups + 16 <= Net::CTRL, "control block");
 
   if (threadIdx.x == 0) {
     for (int w = 0; w < kGroups; ++w) {
@@ -190,6 +203,7 @@ __global__ void __launch_bounds__(Net::THREADS) __maxnreg__(Net::MAXREG)
       mbar_init(bar_c0 + 8 * w, 1);
       mbar_init(bar_c + 8 * w, 1);
       mbar_init(bar_a + 8 * w, 4);
+      mbar_init(bar_a2 + 8 * w, 4);
       mbar_init(bar_drain + 8 * w, 1);
     }
     *abort_flag = 0;
@@ -225,7 +239,7 @@ __global__ void __launch_bounds__(Net::THREADS) __maxnreg__(Net::MAXREG)
     const int w = warp >> 2, par = w & 1;
     // the two regions of this warp's lanes, XORed by 64 columns
     const uint32_t t_base = tmem + (static_cast<uint32_t>((warp & 3) * 32) << 16) + static_cast<uint32_t>(w * 2 * N);
-    const uint32_t my_c0 = bar_c0 + 8 * w, my_c = bar_c + 8 * w, my_a = bar_a + 8 * w;
+    const uint32_t my_c0 = bar_c0 + 8 * w, my_c = bar_c + 8 * w, my_a = bar_a + 8 * w, my_a2 = bar_a2 + 8 * w;
     uint32_t c0_phase = 0, c_phase = 0, reg = 0;
 
     for (long long seg = t_begin; seg < t_end;) {
@@ -262,14 +276,16 @@ __global__ void __launch_bounds__(Net::THREADS) __maxnreg__(Net::MAXREG)
           if (k == 0) c0_phase ^= 1u;
           else c_phase ^= 1u;
           tc_fence_after();
-          epilogue<Net>(t_base + reg);
+          epilogue<Net>(t_base + reg, [&](bool first) {
+            tc_fence_before();
+            __syncwarp();
+            // p.test_fault (tests of the bounded waits only): one warp of each
+            // of CTA 0's groups withholds its first arrival
+            if (lane == 0 &&
+                !(p.test_fault && blockIdx.x == 0 && (warp & 3) == 0 && seg == t_begin && i == 0 && k == 0 && first))
+              mbar_arrive(first ? my_a : my_a2);
+          });
           reg ^= N;
-          tc_fence_before();
-          __syncwarp();
-          // p.test_fault (tests of the bounded waits only): one warp of each
-          // of CTA 0's groups withholds its first arrival
-          if (lane == 0 && !(p.test_fault && blockIdx.x == 0 && (warp & 3) == 0 && seg == t_begin && i == 0 && k == 0))
-            mbar_arrive(my_a);
         }
         if (!ok) break;
         ok = wait(my_c, c_phase);
@@ -345,7 +361,7 @@ __global__ void __launch_bounds__(Net::THREADS) __maxnreg__(Net::MAXREG)
     constexpr uint32_t id_hidden = idesc_f16(128, N), id_out = idesc_f16(128, 16);
     constexpr uint64_t kStep = 256 >> 4;  // one K step (16 fp16)
     const uint32_t my_ff = bar_ff + 8 * w, my_fe = bar_fe + 8 * w, my_c0 = bar_c0 + 8 * w, my_c = bar_c + 8 * w,
-                   my_a = bar_a + 8 * w;
+                   my_a = bar_a + 8 * w, my_a2 = bar_a2 + 8 * w;
     uint32_t a_phase = 0, ff_phase = 0, reg = 0;
     // layer 0 of the group's next tile into region reg
     auto first_layer = [&]() -> bool {
@@ -374,27 +390,33 @@ __global__ void __launch_bounds__(Net::THREADS) __maxnreg__(Net::MAXREG)
       bool ok = tiles > 0 && first_layer();
       for (int i = 0; i < tiles && ok; ++i) {
         for (int k = 1; k < NL; ++k) {
-          ok = wait(my_a, a_phase);
-          if (!ok) break;
-          a_phase ^= 1u;
           const uint32_t ta = t_base + reg, d = t_base + (reg ^ N);
           reg ^= N;
-          if (elect_one()) {
-            tc_fence_after();
-            const bool out_layer = k == NL - 1;
-            const uint64_t db = out_layer ? dBO : dBH + (k - 1) * (Net::BH_BYTES >> 4);
-            const uint32_t id = out_layer ? id_out : id_hidden;
-            if (!out_layer) mma_f16(d, dONES, dBB + k * (Net::BB_BYTES >> 4), id, 0);  // bias: [1 0..0] x [b 0..0]
-            // the lo terms first: each MMA rounds the running sum, which is
-            // small until the hi terms come
+          const bool out_layer = k == NL - 1;
+          const uint64_t db = out_layer ? dBO : dBH + (k - 1) * (Net::BH_BYTES >> 4);
+          const uint32_t id = out_layer ? id_out : id_hidden;
 #pragma unroll
-            for (int s = 0; s < N / 16; ++s)
-              mma_f16_ta(d, ta + 16 * s + 8, db + s * kStep, id, s > 0 || !out_layer);
+          for (int part = 0; part < 2; ++part) {
+            ok = wait(part == 0 ? my_a : my_a2, a_phase);
+            if (!ok) break;
+            if (elect_one()) {
+              tc_fence_after();
+              // bias: [1 0..0] x [b 0..0]
+              if (part == 0 && !out_layer) mma_f16(d, dONES, dBB + k * (Net::BB_BYTES >> 4), id, 0);
+              // the lo terms first: each MMA rounds the running sum, which is
+              // small until the hi terms come
 #pragma unroll
-            for (int s = 0; s < N / 16; ++s) mma_f16_ta(d, ta + 16 * s, db + s * kStep, id, 1);
-            mma_commit(my_c);
+              for (int s = part ? Net::CUT : 0; s < (part ? N / 16 : Net::CUT); ++s)
+                mma_f16_ta(d, ta + 16 * s + 8, db + s * kStep, id, s > 0 || !out_layer);
+#pragma unroll
+              for (int s = part ? Net::CUT : 0; s < (part ? N / 16 : Net::CUT); ++s)
+                mma_f16_ta(d, ta + 16 * s, db + s * kStep, id, 1);
+              if (part == 1) mma_commit(my_c);
+            }
+            __syncwarp();
           }
-          __syncwarp();
+          if (!ok) break;
+          a_phase ^= 1u;
         }
         reg ^= N;  // the region of the output layer's operand, free behind it
         if (ok && i + 1 < tiles) ok = first_layer();
