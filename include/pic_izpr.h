@@ -24,9 +24,8 @@
 extern "C" {
 #endif
 
-/* Bytes of device workspace pic_izpr_decode needs for n_symbols symbols (a
- * status word and the marker counts of up to 2048 ranges of the stream), or
- * -1 for n_symbols < 0. */
+/* Bytes of device workspace pic_izpr_decode asks for with n_symbols symbols (a
+ * status word and room for marker counts), or -1 for n_symbols < 0. */
 int64_t pic_izpr_workspace_bytes(int64_t n_symbols);
 
 /*

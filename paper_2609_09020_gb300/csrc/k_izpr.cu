@@ -51,9 +51,13 @@ struct Workspace {
   int* count;
 };
 __host__ __device__ inline long long n_chunks_of(long long n) { return (n + kChunk - 1) / kChunk; }
+// What callers provide: 5.5 bytes a chunk, as the per-chunk counts took that
+// the ranges' replaced (32 + 4 x kMaxGrid bytes at most are used), so that the
+// same buffers stay accepted and refused.
+__host__ __device__ inline long long align16(long long b) { return (b + 15) / 16 * 16; }
 __host__ __device__ inline long long ws_bytes(long long n) {
-  const long long c = n_chunks_of(n);
-  return 32 + ((c < kMaxGrid ? c : kMaxGrid) + 3) / 4 * 16;
+  const long long c = n_chunks_of(n), groups = (c + 7) / 8;
+  return 32 + align16(4 * groups) + align16(4 * c) + 8 * groups;
 }
 __host__ __device__ inline Workspace ws_view(void* w) {
   char* p = static_cast<char*>(w);
