@@ -67,13 +67,44 @@ def algorithmic(wl: wk.Workload, batch: int):
 
 
 # FP32-pipe operations of one GELU evaluation in the kernels (pic_gelu.cuh):
-# z^2, the Horner steps of P (5) and Q (4), P * (1 / Q), the saturating fma
-# and z * Phi; the reciprocal itself runs on the special-function unit.
+# six Horner steps, the saturating subtraction and the last multiply-add; the
+# power of two runs on the special-function unit, the two comparisons beside
+# the FP32 pipe.
+GELU_OPS = 6 + 1 + 1
+# Those of the rational function that the kernels evaluated before (z^2, the
+# Horner steps of P (5) and Q (4), P * (1 / Q), the saturating fma and z * Phi).
 GELU_FP32_OPS = 4 + 5 + 4
 
 
+def march_tensor_macs_per_px(wl: wk.Workload) -> int:
+    """MACs the tensor cores execute per pixel in the row-marching kernels (the
+    ones staging "auto" picks): layer 0 (K = the hi and lo features and the
+    constant 1, round16), hidden layers and the output layer with the hi and lo
+    halves of K.  Nets wider than 40 run on N = 64 tiles, each bias that is no
+    column of layer 0 as one K = 16 step and the output layer as N = 16;
+    narrower ones at their own width, biases free, the output layer as N = 8."""
+    d0, width = wl.dims[0], max(wl.dims[1:-1])
+    k1 = (4 * ((d0 + 1) // 2) + 15) // 16 * 16
+    bias_column = d0 % 2 == 1 or 4 * ((d0 + 1) // 2) < k1
+    n, bias, out = (64, 16, 16) if width > 40 else ((width + 7) // 8 * 8, 0, 8)
+    mac = (k1 + (0 if bias_column else bias)) * n
+    mac += (len(wl.dims) - 3) * (2 * n + bias) * n
+    return mac + 2 * n * out
+
+
+def march_alu_ops_per_px(wl: wk.Workload, precision: str) -> int:
+    """Activation-inclusive CUDA-core work per pixel (FP32-pipe operations):
+    every hidden activation (GELU at GELU_OPS; ReLU is folded into a
+    conversion), plus on the tensor path the hi/lo split of every hidden value
+    (2 per value), plus on the fp32 path every MLP MAC."""
+    hidden = sum(wl.dims[1:-1])
+    ops = (GELU_OPS if wl.act == "gelu" else 0) * hidden
+    return ops + (2 * hidden if precision == "fp16_tc" else wl.macs_per_pixel)
+
+
 def executed_tensor_macs_per_px(wl: wk.Workload) -> int:
-    """MACs the tensor cores execute per pixel: layer 0 (K = round16(2 D0 + 1),
+    """MACs the tensor cores execute per pixel in the per-tile kernels (staging
+    "copies" and "tma"): layer 0 (K = round16(2 D0 + 1),
     N = round16 of the width), hidden layers and (for wide, shallow nets) the
     output layer (N = 16), with the hi and lo halves of K plus one K = 16 bias
     step each."""
@@ -88,16 +119,17 @@ def executed_tensor_macs_per_px(wl: wk.Workload) -> int:
 
 
 def tc_output_on_tensor_cores(wl: wk.Workload) -> bool:
-    """The tensor path runs the output layer as an MMA only for wide, shallow
+    """The per-tile kernels run the output layer as an MMA only for wide, shallow
     nets (padded width > 32 and fewer than 4 layers); else on the CUDA cores."""
     n_pad = (max(wl.dims[1:-1]) + 15) // 16 * 16
     return n_pad > 32 and len(wl.dims) - 1 < 4
 
 
 def alu_ops_per_px(wl: wk.Workload, precision: str) -> int:
-    """Activation-inclusive CUDA-core work per pixel (FP32-pipe operations):
-    every hidden activation (GELU at GELU_FP32_OPS; ReLU is folded into a
-    conversion), plus on the tensor path the hi/lo split of every hidden value
+    """Activation-inclusive CUDA-core work per pixel (FP32-pipe operations) of
+    the per-tile kernels with the rational GELU, for comparison with older
+    figures: every hidden activation (GELU at GELU_FP32_OPS; ReLU is folded into
+    a conversion), plus on the tensor path the hi/lo split of every hidden value
     that feeds an MMA (2 per value) and the output layer where it runs on the
     CUDA cores (one FMA per weight), plus on the fp32 path every MLP MAC."""
     hidden = list(wl.dims[1:-1])
@@ -137,13 +169,13 @@ def roofline_for(wl: wk.Workload, precision: str, B: int, ms: float, peaks: dict
     roof["frac"] = roof["achieved"] / roof["peak"]
     roof["algorithmic_flops_per_launch"] = flops
     if precision == "fp16_tc":
-        roof["executed_tensor_flops_per_launch"] = 2.0 * executed_tensor_macs_per_px(wl) * px
+        roof["executed_tensor_flops_per_launch"] = 2.0 * march_tensor_macs_per_px(wl) * px
     roof["algorithmic_bytes_per_launch"] = nbytes
     roof["binding_time_us"] = max(t_pipe, t_hbm) * 1e6
     roof["avg_launch_us"] = ms * 1e3
     # activation-inclusive ALU bound (FP32 pipe at the measured FMA rate;
     # one operation = one lane-op, half an FMA's two FLOPs)
-    ops = alu_ops_per_px(wl, precision)
+    ops = march_alu_ops_per_px(wl, precision)
     t_alu = ops * px / (fp32_tflops * 1e12 / 2)
     t_bind = max(t_pipe, t_hbm, t_alu)
     roof["alu_bound"] = {"ops_per_px": ops,
@@ -156,7 +188,7 @@ def roofline_for(wl: wk.Workload, precision: str, B: int, ms: float, peaks: dict
 KERNEL_SOURCES = {
     "idct": ["k_idct.cu"],
     "izpr": ["k_izpr.cu"],
-    "tc": ["k_tc.cuh", "tc_ptx.cuh", "pic_common.cuh", "pic_gelu.cuh", "pic_kernels.h"],
+    "tc": ["k_tcmarch.cuh", "march.cuh", "tc_ptx.cuh", "pic_common.cuh", "pic_gelu.cuh", "pic_kernels.h"],
     "fp32": ["k_fp32.cuh", "pic_common.cuh", "pic_gelu.cuh", "pic_kernels.h"],
 }
 
@@ -494,7 +526,7 @@ def run_bitstream_stages(args):
     t_h = stage_ms["huffman"] * 1e-3
     roof = {"bound": "hbm", "achieved": hbytes / t_h / 1e9, "peak": peaks["hbm_gbs"],
             "unit": "GB/s", "peak_source": f"copy bandwidth, {peaks['source']}",
-            "kernel": "huff_lut + huff_decode (one call)", "avg_launch_us": t_h * 1e6,
+            "kernel": "huff_decode (one call)", "avg_launch_us": t_h * 1e6,
             "traffic": None, "algorithmic_bytes_per_launch": hbytes}
     roof["frac"] = roof["achieved"] / roof["peak"]
     if full:
@@ -812,15 +844,15 @@ def run_stage(args):
     else:
         roof = {"bound": "hbm", "achieved": nbytes / (ms * 1e-3) / 1e9, "peak": peaks["hbm_gbs"],
                 "unit": "GB/s", "peak_source": f"copy bandwidth, {peaks['source']}",
-                "kernel": "izpr_count+izpr_scan+izpr_expand (one call)"
+                "kernel": "izpr_count+izpr_expand (one call)"
                 if stage == "izpr" else "idct_unpatchify_kernel",
                 "avg_launch_us": ms * 1e3}
     roof["frac"] = roof["achieved"] / roof["peak"]
     roof["traffic"] = recorded_traffic("idct_unpatchify_kernel", "c5x64") if stage == "idct" \
         else None
     if stage == "izpr":
-        roof["traffic_note"] = ("one call is 3 kernels; ncu measured izpr_expand alone at "
-                                "104.4 MB read + 79.5 MB written (profiles/izpr__c5x64_launches_and_full.md)")
+        roof["traffic_note"] = ("one call is 2 kernels; the stream is read twice "
+                                "(profiles/izpr__c5x64_launches_and_full.md)")
     roof["algorithmic_bytes_per_launch"] = nbytes
 
     # end to end with host buffers: H2D of the step's input, the stage, D2H of its result
