@@ -452,7 +452,7 @@ __device__ __forceinline__ void advance_tile(int& yy, int& xx, int tpr) {
   }
 }
 
-template <class Net, bool FL, bool TMA>
+template <class Net, bool TMA>
 __global__ void __launch_bounds__(Net::THREADS) __maxnreg__(Net::MAXREG)
     tc_decode_kernel(const DecodeParams p, const __grid_constant__ TmaParams tp) {
   constexpr int N = Net::N, NL = Net::NL, C = Net::C, L = Net::L, D0 = Net::D0, NWG = Net::NWG;
@@ -564,7 +564,7 @@ __global__ void __launch_bounds__(Net::THREADS) __maxnreg__(Net::MAXREG)
         const int32_t* lat = p.latents + b * p.lat_per_image;
         float step[L];
 #pragma unroll
-        for (int l = 0; l < L; ++l) step[l] = FL ? 1.0f : __ldg(p.steps + b * L + l);
+        for (int l = 0; l < L; ++l) step[l] = __ldg(p.steps + b * L + l);
 
         // This thread's column items: level, column, and the level's geometry.
         int it_l[JJ], it_i[JJ], it_W[JJ], it_H[JJ];
@@ -662,7 +662,7 @@ __global__ void __launch_bounds__(Net::THREADS) __maxnreg__(Net::MAXREG)
             if (l > 0) {
               const float beta = it_beta[j];  // set by the prefetch of this tile
               const int t0 = stage[(C + 2 * j) * kTile + r], t1 = stage[(C + 2 * j + 1) * kTile + r];
-              colbuf[sr + SEG * j] = step[l] * lat_lerp<FL>(t0, t1, beta);
+              colbuf[sr + SEG * j] = step[l] * lat_lerp<false>(t0, t1, beta);
             }
           }
           if constexpr (TMA || SEG == kTile) {
@@ -684,9 +684,9 @@ __global__ void __launch_bounds__(Net::THREADS) __maxnreg__(Net::MAXREG)
             if constexpr (TMA) {
               const unsigned sc = img_word + static_cast<unsigned>(c * plane + y * p.W + x0);
               const int* slot = reinterpret_cast<const int*>(tbuf + (k & 1) * Net::TBUF_BYTES + TS::off(c));
-              f[c] = step[0] * lat_value<FL>(slot[(sc & 3u) + r]);
+              f[c] = step[0] * lat_value<false>(slot[(sc & 3u) + r]);
             } else {
-              f[c] = step[0] * lat_value<FL>(stage[c * kTile + r]);
+              f[c] = step[0] * lat_value<false>(stage[c * kTile + r]);
             }
           }
 #pragma unroll
@@ -993,14 +993,14 @@ __global__ void __launch_bounds__(Net::THREADS) __maxnreg__(Net::MAXREG)
   }
 }
 
-template <int C, int NL, int D0, int N, int ACT, int NWG, bool FL, bool TMA = false, bool LO8 = false,
+template <int C, int NL, int D0, int N, int ACT, int NWG, bool TMA = false, bool LO8 = false,
           int NR = N>
 KernelInfo make_tc(const char* name, const int* dims) {
   using Net = TcNet<C, NL, D0, N, ACT, NWG, LO8, NR>;
   KernelInfo k{};
   k.name = name;
   k.precision = LO8 ? 2 : 1;
-  k.latent_format = FL ? 1 : 0;
+  k.latent_format = 0;
   k.C = C;
   k.n_layers = NL;
   for (int i = 0; i <= NL; ++i) k.dims[i] = dims[i];
@@ -1010,7 +1010,7 @@ KernelInfo make_tc(const char* name, const int* dims) {
   k.tile_px = kTile;
   k.smem_bytes = TMA ? Net::SMEM_TMA : Net::SMEM;
   k.tma = TMA ? 1 : 0;
-  k.fn = reinterpret_cast<const void*>(&tc_decode_kernel<Net, FL, TMA>);
+  k.fn = reinterpret_cast<const void*>(&tc_decode_kernel<Net, TMA>);
   return k;
 }
 
