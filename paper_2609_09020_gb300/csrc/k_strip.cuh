@@ -12,10 +12,11 @@
 // tcgen05's rate (8.2 cycles per m16n8k16 and sub-partition) and each one
 // takes about 6 cycles of the FMA pipe besides, so its share grows with the
 // square of the width; up to 40 it pays.  64 images of 768x512, the per-tile
-// kernel's time first: 8-8-8-8-3 573 -> 274 us, 8-16-16-16-3 636 -> 367 us,
-// 8-32-32-32-3 790 -> 756 us; one 7-40-40-3 GELU image and one 256x256
-// 4-16-16-3 image are within 2 % of it.  Bound by issue and latency: 306
-// warp instructions per 32 pixels of the 16-wide net at 0.52 a cycle.
+// kernel's time first: 8-8-8-8-3 573 -> 259 us, 8-16-16-16-3 636 -> 354 us,
+// 8-32-32-32-3 790 -> 743 us; one 7-40-40-3 GELU image and one 256x256
+// 4-16-16-3 image are within 2 % of it.  Bound by issue, latency and the L1
+// data pipe: 306 warp instructions per 32 pixels of the 16-wide net at 0.57 a
+// cycle, and 78 % of the pipe's rate before the weights moved to registers.
 //
 // Precision is that of the tcgen05 kernels: fp16 weights as given, every
 // activation as hi + lo fp16 terms (~22 bits), fp32 accumulation; biases
@@ -43,6 +44,12 @@ struct StripNet {
   static constexpr int WH_WORDS = frag_words(J, J);
   static constexpr int WO_WORDS = frag_words(1, J);
   static constexpr int OFF_H = W1_WORDS, OFF_O = OFF_H + HID * WH_WORDS, OFF_B = OFF_O + WO_WORDS;
+  // Weight fragments, two registers a lane each.  Up to width 16 they fit into
+  // registers for an image's rows (24 images of 768x512: width 8 109 -> 104
+  // us, width 16 144 -> 139.5 us, of shared memory's 102 wavefronts a row 14);
+  // the next wider net has 22, which spill.
+  static constexpr int FRAGS = OFF_B / 64;
+  static constexpr bool HELD = FRAGS <= 8;
   // bias tables (load_bias): layer 0 (BIASCOL nets: zeros), hidden layers, output
   static constexpr int B_WORDS = ((1 + HID) * J + 1) * 16;
   static constexpr int PARAMS = N * (F::D0 + 1) + HID * N * (N + 1) + 3 * (N + 1);
@@ -87,9 +94,9 @@ __device__ __forceinline__ void load_weights_strip(uint32_t* sm, const __half* w
 
 // d = A B + bias for both pixel halves, A the hi and lo fragments of the previous
 // layer's J tiles (blocks 0 .. J-1 hi, J .. 2J-1 lo, both against the same
-// weights), B the fragments at `wf` (JO output tiles of J blocks).
-template <int J, int JO>
-__device__ __forceinline__ void layer(const uint32_t* wf, const float* bias4, int lane, const uint32_t (&hi)[2][J][2],
+// weights), B the fragments from the f0-th on (JO output tiles of J blocks).
+template <int J, int JO, class Frag>
+__device__ __forceinline__ void layer(const Frag& frag, int f0, const float* bias4, int lane, const uint32_t (&hi)[2][J][2],
                                       const uint32_t (&lo)[2][J][2], float (&d)[2][JO][4]) {
   constexpr int NB2 = (J + 1) / 2;
 #pragma unroll
@@ -99,7 +106,7 @@ __device__ __forceinline__ void layer(const uint32_t* wf, const float* bias4, in
     load_bias(bias4, j, lane, c);
 #pragma unroll
     for (int i2 = 0; i2 < NB2; ++i2) {
-      const uint2 v = *reinterpret_cast<const uint2*>(wf + (j * NB2 + i2) * 64 + 2 * lane);
+      const uint2 v = frag(f0 + j * NB2 + i2);
       b[2 * i2] = v.x;
       b[2 * i2 + 1] = v.y;
     }
@@ -172,6 +179,15 @@ __global__ void __launch_bounds__(kStripThreads, Net::MINB) strip_decode_kernel(
     __syncthreads();
     load_weights_strip<Net>(sw, reinterpret_cast<const __half*>(smem + Net::OFF_RAW) + raw_skip(w), threadIdx.x);
     __syncthreads();
+    uint2 held[Net::HELD ? Net::FRAGS : 1];
+    if constexpr (Net::HELD) {
+#pragma unroll
+      for (int f = 0; f < Net::FRAGS; ++f) held[f] = *reinterpret_cast<const uint2*>(sw + f * 64 + 2 * lane);
+    }
+    auto frag = [&](int f) {
+      if constexpr (Net::HELD) return held[f];
+      else return *reinterpret_cast<const uint2*>(sw + f * 64 + 2 * lane);
+    };
     for (bool started = true; t < te; started = false) {
       if (!started) {
         tc::cp_async_wait_all();
@@ -188,7 +204,7 @@ __global__ void __launch_bounds__(kStripThreads, Net::MINB) strip_decode_kernel(
           load_a<F>(mine + Net::OFF_A, lane, 1, s, a[1]);
 #pragma unroll
           for (int j = 0; j < J; ++j) {
-            const uint2 v = *reinterpret_cast<const uint2*>(sw + (j * (Net::NB1 / 2) + s) * 64 + 2 * lane);
+            const uint2 v = frag(j * (Net::NB1 / 2) + s);
             if (s == 0) {
               float c[4] = {0.0f, 0.0f, 0.0f, 0.0f};
               if constexpr (!F::BIASCOL) load_bias(bias, j, lane, c);
@@ -204,11 +220,11 @@ __global__ void __launch_bounds__(kStripThreads, Net::MINB) strip_decode_kernel(
 #pragma unroll
         for (int h = 0; h < HID; ++h) {
           split_acc<Net::ACT, J>(d, hi, lo);
-          layer<J, J>(sw + Net::OFF_H + h * Net::WH_WORDS, bias + (1 + h) * 16 * J, lane, hi, lo, d);
+          layer<J, J>(frag, (Net::OFF_H + h * Net::WH_WORDS) / 64, bias + (1 + h) * 16 * J, lane, hi, lo, d);
         }
         split_acc<Net::ACT, J>(d, hi, lo);
         float o[2][1][4];
-        layer<J, 1>(sw + Net::OFF_O, bias + (1 + HID) * 16 * J, lane, hi, lo, o);
+        layer<J, 1>(frag, Net::OFF_O / 64, bias + (1 + HID) * 16 * J, lane, hi, lo, o);
         const float rgb[2][4] = {{o[0][0][0], o[0][0][1], o[0][0][2], o[0][0][3]},
                                  {o[1][0][0], o[1][0][1], o[1][0][2], o[1][0][3]}};
         put_rgb(mine + Net::OFF_OUT, lane, rgb);
