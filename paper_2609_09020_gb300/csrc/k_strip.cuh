@@ -236,6 +236,7 @@ __global__ void __launch_bounds__(kStripThreads, Net::MINB) strip_decode_kernel(
     }
     seg = seg_end;
   }
+  tc::cp_async_wait_all();  // copies still in flight land before shared memory goes
 }
 
 template <int L, int C, int NL, int N, int ACT, bool FL = false>
