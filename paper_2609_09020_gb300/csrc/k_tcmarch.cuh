@@ -19,9 +19,13 @@
 // 16 accumulator columns it reads by the 8 columns of hi pairs and 8 of lo
 // pairs made from them, so a layer's operand lies where its input's
 // accumulator was, and the layer accumulates into the other region.  The
-// next tile's layer 0 (operand from shared memory) can therefore be queued
-// right behind a tile's output layer, into the region whose operand that
-// layer reads; its latency disappears behind the output layer's.
+// next tile's layer 0 (operand from shared memory) goes into the region whose
+// operand a tile's last layer reads, as soon as that layer is complete; its
+// latency disappears behind the decoding warps' RGB.  (Queued right behind the
+// last layer, without the wait, it would rest on issue order alone, which
+// tensor-memory MMAs keep only with the same accumulator and shape; the wait
+// costs 1 %: 64 images of 768x512 660 -> 668 us, 16-64-64-64-3 at 3840x2160
+// 789 -> 795 us.)
 //
 // What bounds it: the chain of a tile's two (or more) remaining round trips
 // with four tiles in flight -- tensor memory holds no more -- and, next to
@@ -362,7 +366,7 @@ __global__ void __launch_bounds__(Net::THREADS) __maxnreg__(Net::MAXREG)
     constexpr uint64_t kStep = 256 >> 4;  // one K step (16 fp16)
     const uint32_t my_ff = bar_ff + 8 * w, my_fe = bar_fe + 8 * w, my_c0 = bar_c0 + 8 * w, my_c = bar_c + 8 * w,
                    my_a = bar_a + 8 * w, my_a2 = bar_a2 + 8 * w;
-    uint32_t a_phase = 0, ff_phase = 0, reg = 0;
+    uint32_t a_phase = 0, c_phase = 0, ff_phase = 0, reg = 0;
     // layer 0 of the group's next tile into region reg
     auto first_layer = [&]() -> bool {
       if (!wait(my_ff, ff_phase)) return false;
@@ -417,9 +421,10 @@ __global__ void __launch_bounds__(Net::THREADS) __maxnreg__(Net::MAXREG)
           }
           if (!ok) break;
           a_phase ^= 1u;
+          c_phase ^= 1u;
         }
-        reg ^= N;  // the region of the output layer's operand, free behind it
-        if (ok && i + 1 < tiles) ok = first_layer();
+        reg ^= N;  // the region of the last layer's operand, free once that layer is complete
+        if (ok && i + 1 < tiles) ok = wait(my_c, c_phase ^ 1u) && first_layer();
       }
       seg = seg_end;
     }
