@@ -18,9 +18,10 @@
 // data pipe: 306 warp instructions per 32 pixels of the 16-wide net at 0.57 a
 // cycle, and 78 % of the pipe's rate before the weights moved to registers.
 //
-// Precision is that of the tcgen05 kernels: fp16 weights as given, every
-// activation as hi + lo fp16 terms (~22 bits), fp32 accumulation; biases
-// enter as the accumulators' start values or, where operand A has room, as
+// Precision is that of the per-tile tcgen05 kernels: fp16 weights as given, every
+// activation that an MMA reads as hi + lo fp16 terms (~22 bits, values below
+// 131,008), fp32 accumulation, and the output layer of all but 7-40-40-3 on
+// fp32 hidden values; biases enter as the accumulators' start values or, where operand A has room, as
 // the weight of a constant-1 column.
 #pragma once
 
@@ -33,6 +34,8 @@ namespace {
 constexpr int kStripWarps = 4;
 constexpr int kStripThreads = 32 * kStripWarps;
 
+constexpr int kOutRow = 12;  // output weights of a lane's two neurons of a tile: 2 x 3, each twice
+
 template <int L_, int C_, int NL_, int N_, int ACT_>
 struct StripNet {
   static constexpr int L = L_, C = C_, NL = NL_, N = N_, ACT = ACT_;
@@ -42,20 +45,26 @@ struct StripNet {
   static constexpr int HID = NL - 2;         // hidden x hidden layers
   static constexpr int W1_WORDS = frag_words(J, NB1);
   static constexpr int WH_WORDS = frag_words(J, J);
-  static constexpr int WO_WORDS = frag_words(1, J);
+  // Output layer in fp32 (output_layer), as the per-tile kernels have it for
+  // nets at most 32 wide or with four layers; 7-40-40-3 alone is left, whose
+  // hidden values go to the tensor pipe as pairs there too (24 images of
+  // 768x512: 476 us, 490 in fp32).
+  static constexpr bool OUT_FP32 = N <= 32 || NL >= 4;
+  static constexpr int WO_WORDS = OUT_FP32 ? 4 * J * kOutRow + 4 : frag_words(1, J);
   static constexpr int OFF_H = W1_WORDS, OFF_O = OFF_H + HID * WH_WORDS, OFF_B = OFF_O + WO_WORDS;
   // Weight fragments, two registers a lane each.  Up to width 16 they fit into
   // registers for an image's rows (24 images of 768x512: width 8 109 -> 104
-  // us, width 16 144 -> 139.5 us, of shared memory's 102 wavefronts a row 14);
-  // the next wider net has 22, which spill.
-  static constexpr int FRAGS = OFF_B / 64;
+  // us, width 16 144 -> 139.5 us with the output layer among them, of shared
+  // memory's 102 wavefronts a row 14); the next wider net has 20, which spill.
+  static constexpr int FRAGS = OFF_O / 64;
   static constexpr bool HELD = FRAGS <= 8;
-  // bias tables (load_bias): layer 0 (BIASCOL nets: zeros), hidden layers, output
-  static constexpr int B_WORDS = ((1 + HID) * J + 1) * 16;
+  // bias tables (load_bias): layer 0 (BIASCOL nets: zeros), hidden layers, output (unless in fp32)
+  static constexpr int B_WORDS = ((1 + HID) * J + (OUT_FP32 ? 0 : 1)) * 16;
   static constexpr int PARAMS = N * (F::D0 + 1) + HID * N * (N + 1) + 3 * (N + 1);
   static constexpr int OFF_RAW = round_to((OFF_B + B_WORDS) * 4, 128);  // the weights as given (copy_raw)
   static constexpr int W_BYTES = OFF_RAW + raw_bytes(PARAMS);
-  static constexpr int OFF_A = F::FEAT_BYTES, OFF_OUT = OFF_A + F::A_BYTES, WARP_BYTES = OFF_OUT + kOutBytes;
+  static constexpr int OFF_A = F::FEAT_BYTES, OFF_OUT = OFF_A + F::A_BYTES;
+  static constexpr int WARP_BYTES = OFF_OUT + (OUT_FP32 ? 0 : kOutBytes);
   static constexpr int SMEM = W_BYTES + kStripWarps * WARP_BYTES;
   // CTAs per SM: five hide more latency where their 96 registers do (width
   // 8: 301 -> 274 us); wider nets spill there (width 16 equal, 32 and 40
@@ -86,10 +95,19 @@ __device__ __forceinline__ void load_weights_strip(uint32_t* sm, const __half* w
               [&](int n) { return __half2float(p[N * N + n]); });
     p += N * N + N;
   }
-  fill_frags<1, Net::J>(sm + Net::OFF_O, tid, kStripThreads,
-                        [&](int n, int k) { return n < 3 ? p[n * N + k] : zero; });
-  fill_bias(bias + (1 + Net::HID) * 16 * Net::J, 1, tid, kStripThreads,
-            [&](int n) { return n < 3 ? __half2float(p[3 * N + n]) : 0.0f; });
+  if constexpr (Net::OUT_FP32) {  // [tile j][t][neuron 8j + 2t, the next][r r g g b b], then the biases
+    float* wo = reinterpret_cast<float*>(sm + Net::OFF_O);
+    for (int e = tid; e < 4 * Net::J * kOutRow; e += kStripThreads) {
+      const int jt = e / kOutRow, q = e - jt * kOutRow, h = q / 6;
+      wo[e] = __half2float(p[(q - 6 * h) / 2 * N + 2 * jt + h]);
+    }
+    if (tid < 3) wo[4 * Net::J * kOutRow + tid] = __half2float(p[3 * N + tid]);
+  } else {
+    fill_frags<1, Net::J>(sm + Net::OFF_O, tid, kStripThreads,
+                          [&](int n, int k) { return n < 3 ? p[n * N + k] : zero; });
+    fill_bias(bias + (1 + Net::HID) * 16 * Net::J, 1, tid, kStripThreads,
+              [&](int n) { return n < 3 ? __half2float(p[3 * N + n]) : 0.0f; });
+  }
 }
 
 // d = A B + bias for both pixel halves, A the hi and lo fragments of the previous
@@ -135,6 +153,48 @@ __device__ __forceinline__ void split_acc(const float (&d)[2][J][4], uint32_t (&
       for (int h = 0; h < 2; ++h) act_split<ACT>(d[m][j][2 * h], d[m][j][2 * h + 1], hi[m][j][h], lo[m][j][h]);
 }
 
+// Activation and output layer in fp32: the hidden values stay as wide as the
+// accumulators they come from (an fp16 pair would end at 131,008 and lose bits
+// below 2^-3).  Each lane sums over its neurons (8j + 2t, 8j + 2t + 1 with t =
+// lane % 4) for its four pixels, in pairs of the two pixel rows of a fragment;
+// two exchanges add up the four lanes' sums and leave lane 4g + t with pixel
+// out_pixel(lane) = 16 (t & 1) + 8 (t >> 1) + g of the strip.  Against split
+// pairs and one MMA a tile, which cost no exchange, 24 images of 768x512:
+// 8-8-8-8-3 104 -> 112 us, 8-16-16-16-3 143 -> 159 us, 8-32-32-32-3 285 -> 297
+// us.  The exchanges are 8 us of it; weights in registers, sums in pairs of
+// neurons, or the exchanges finished beside the next row's features are within
+// 2 % of this.
+__device__ __forceinline__ int out_pixel(int lane) { return 16 * (lane & 1) + 4 * (lane & 2) + (lane >> 2); }
+
+template <class Net>
+__device__ __forceinline__ void output_layer(const float* wo, int lane, const float (&d)[2][Net::J][4], float (&rgb)[3]) {
+  constexpr int J = Net::J;
+  auto act = [](float a, float b) {
+    if constexpr (Net::ACT == ACT_GELU) return gelu_approx2(pack2(a, b));
+    else return pack2(fmaxf(a, 0.0f), fmaxf(b, 0.0f));
+  };
+  unsigned long long s[2][3];
+#pragma unroll
+  for (int j = 0; j < J; ++j) {
+    const ulonglong2* w = reinterpret_cast<const ulonglong2*>(wo + (4 * j + (lane & 3)) * kOutRow);
+    const ulonglong2 w0 = w[0], w1 = w[1], w2 = w[2];
+#pragma unroll
+    for (int m = 0; m < 2; ++m) {
+      const unsigned long long a = act(d[m][j][0], d[m][j][2]), b = act(d[m][j][1], d[m][j][3]);
+      s[m][0] = fma2(w1.y, b, j == 0 ? mul2(w0.x, a) : fma2(w0.x, a, s[m][0]));
+      s[m][1] = fma2(w2.x, b, j == 0 ? mul2(w0.y, a) : fma2(w0.y, a, s[m][1]));
+      s[m][2] = fma2(w2.y, b, j == 0 ? mul2(w1.x, a) : fma2(w1.x, a, s[m][2]));
+    }
+  }
+  const float* bias = wo + 4 * J * kOutRow;
+#pragma unroll
+  for (int o = 0; o < 3; ++o) {
+    const unsigned long long keep = lane & 1 ? s[1][o] : s[0][o], send = lane & 1 ? s[0][o] : s[1][o];
+    const float2 v = unpack2(add2(keep, __shfl_xor_sync(0xffffffffu, send, 1)));
+    rgb[o] = (lane & 2 ? v.y : v.x) + __shfl_xor_sync(0xffffffffu, lane & 2 ? v.x : v.y, 2) + bias[o];
+  }
+}
+
 template <class Net, bool FL>
 __global__ void __launch_bounds__(kStripThreads, Net::MINB) strip_decode_kernel(const DecodeParams p) {
   using F = typename Net::F;
@@ -142,6 +202,7 @@ __global__ void __launch_bounds__(kStripThreads, Net::MINB) strip_decode_kernel(
   extern __shared__ __align__(128) uint8_t smem[];
   uint32_t* const sw = reinterpret_cast<uint32_t*>(smem);
   const float* const bias = reinterpret_cast<const float*>(sw + Net::OFF_B);
+  const float* const wo = reinterpret_cast<const float*>(sw + Net::OFF_O);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t mine = tc::smem_addr(smem) + Net::W_BYTES + warp * Net::WARP_BYTES;
   Strip<Net::L, Net::C, FL> st;
@@ -222,15 +283,21 @@ __global__ void __launch_bounds__(kStripThreads, Net::MINB) strip_decode_kernel(
           split_acc<Net::ACT, J>(d, hi, lo);
           layer<J, J>(frag, (Net::OFF_H + h * Net::WH_WORDS) / 64, bias + (1 + h) * 16 * J, lane, hi, lo, d);
         }
-        split_acc<Net::ACT, J>(d, hi, lo);
-        float o[2][1][4];
-        layer<J, 1>(frag, Net::OFF_O / 64, bias + (1 + HID) * 16 * J, lane, hi, lo, o);
-        const float rgb[2][4] = {{o[0][0][0], o[0][0][1], o[0][0][2], o[0][0][3]},
-                                 {o[1][0][0], o[1][0][1], o[1][0][2], o[1][0][3]}};
-        put_rgb(mine + Net::OFF_OUT, lane, rgb);
-        float cr, cg, cb;
-        get_rgb(mine + Net::OFF_OUT, lane, cr, cg, cb);
-        write_rgb(p, out_img, b, y0 + r, st.x, cr, cg, cb);
+        float rgb[3];
+        int x = st.x;
+        if constexpr (Net::OUT_FP32) {
+          output_layer<Net>(wo, lane, d, rgb);
+          x = col * 32 + out_pixel(lane);
+        } else {
+          split_acc<Net::ACT, J>(d, hi, lo);
+          float o[2][1][4];
+          layer<J, 1>(frag, Net::OFF_O / 64, bias + (1 + HID) * 16 * J, lane, hi, lo, o);
+          const float both[2][4] = {{o[0][0][0], o[0][0][1], o[0][0][2], o[0][0][3]},
+                                    {o[1][0][0], o[1][0][1], o[1][0][2], o[1][0][3]}};
+          put_rgb(mine + Net::OFF_OUT, lane, both);
+          get_rgb(mine + Net::OFF_OUT, lane, rgb[0], rgb[1], rgb[2]);
+        }
+        write_rgb(p, out_img, b, y0 + r, x, rgb[0], rgb[1], rgb[2]);
       }
       t += rows;
     }

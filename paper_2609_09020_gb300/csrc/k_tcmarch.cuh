@@ -4,8 +4,9 @@
 // row, operands and accumulators in tensor memory.
 //
 // Precision: fp16 weights as given, every activation (feature or hidden
-// value) as hi + lo fp16 terms (hi = truncated, lo = rounded remainder, ~22
-// bits), fp32 accumulation.
+// value) that an MMA reads as hi + lo fp16 terms (hi = truncated, lo = rounded
+// remainder, ~22 bits, values below 131,008), fp32 accumulation; the output
+// layer of nets with four layers on fp32 hidden values.
 //
 // Warps 0-15: four decoding groups of four, one tile at a time each (thread =
 // pixel = tensor-memory lane): accumulator -> activation -> hi/lo split ->
@@ -64,6 +65,14 @@ struct MarchNet {
   static constexpr int L = L_, C = C_, NL = NL_, N = 64, ACT = ACT_;
   using F = FeatLayout<L, C>;
   static constexpr int K1 = F::K1, HID = NL - 2;
+  // Output layer of deep nets in fp32 by the decoding warps (output_layer),
+  // inside the last hidden layer's epilogue: one round trip less, 192 FMAs a
+  // pixel more.  16-64-64-64-3 GELU at 3840x2160: 795 -> 789 us; 8-64-64-64-3,
+  // 24 images of 768x512: 366 -> 383 us; both keep the hidden values' range and
+  // bits, as the per-tile kernels do.  (7-64-64-3 in fp32 measured 762 us with
+  // 657 on the tensor pipe, where the per-tile kernel has it too.)
+  static constexpr bool OUT_FP32 = NL >= 4;
+  static constexpr int MMA_LAYERS = OUT_FP32 ? NL - 1 : NL;
   // An operand is handed to the tensor pipe in two parts, its first 16 columns
   // ahead of the rest: the MMAs of the first part, and the better part of
   // their round trip, run beside the rest of the epilogue.  16-64-64-64-3 GELU
@@ -83,7 +92,7 @@ struct MarchNet {
   // 8 rows x 16 bytes): layer 0's W, the hidden layers' W, the output's W
   // (16 rows, 3 used), and per layer a [rows][16] bias tile (b, 0..0) that
   // meets a constant A tile of rows (1, 0..0).
-  static constexpr int B1_BYTES = N * K1 * 2, BH_BYTES = N * N * 2, BO_BYTES = 16 * N * 2, BB_BYTES = N * 16 * 2;
+  static constexpr int B1_BYTES = N * K1 * 2, BH_BYTES = N * N * 2, BO_BYTES = OUT_FP32 ? 3 * N * 4 : 16 * N * 2, BB_BYTES = N * 16 * 2;
   static constexpr int OFF_ONES = CTRL;
   static constexpr int OFF_B1 = OFF_ONES + 128 * 16 * 2;
   static constexpr int OFF_BH = OFF_B1 + B1_BYTES;
@@ -135,7 +144,15 @@ __device__ __forceinline__ void load_weights_march(uint8_t* smem, const __half* 
                   [&](int n, int k) { return k == 0 ? p[N * N + n] : zero; });
     p += N * N + N;
   }
-  fill_tile<N>(smem + Net::OFF_BO, 16, tid, nthr, [&](int n, int k) { return n < 3 ? p[n * N + k] : zero; });
+  if constexpr (Net::OUT_FP32) {  // four inputs' weights of each colour in turn
+    float* wo = reinterpret_cast<float*>(smem + Net::OFF_BO);
+    for (int e = tid; e < 3 * N; e += nthr) {
+      const int q = e / 12, c = (e - 12 * q) >> 2;
+      wo[e] = __half2float(p[c * N + 4 * q + (e & 3)]);
+    }
+  } else {
+    fill_tile<N>(smem + Net::OFF_BO, 16, tid, nthr, [&](int n, int k) { return n < 3 ? p[n * N + k] : zero; });
+  }
   if (tid < 3) reinterpret_cast<float*>(smem + Net::OFF_BOUT)[tid] = __half2float(p[3 * N + tid]);
 }
 
@@ -175,6 +192,41 @@ __device__ __forceinline__ void epilogue(uint32_t t, Part part_done) {
       tc::tmem_st_wait();
       part_done(c + 1 == Net::CUT);
     }
+  }
+}
+
+// One pixel's accumulator row in region t -> activation and output layer, in
+// fp32 throughout: the hidden values stay as wide as the accumulators they come
+// from (an fp16 pair would end at 131,008 and lose bits below 2^-3).
+template <class Net>
+__device__ __forceinline__ void output_layer(uint32_t t, const float4* wo, float (&rgb)[3]) {
+  uint32_t acc[2][16];
+  unsigned long long s[3] = {0ull, 0ull, 0ull};
+  tc::tmem_ld16(t, acc[0]);
+#pragma unroll
+  for (int c = 0; c < Net::N / 16; ++c) {
+    tc::tmem_ld_wait();
+    if (c + 1 < Net::N / 16) tc::tmem_ld16(t + 16 * (c + 1), acc[(c + 1) & 1]);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      unsigned long long h[2];
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        const float a = __uint_as_float(acc[c & 1][4 * q + 2 * i]), b = __uint_as_float(acc[c & 1][4 * q + 2 * i + 1]);
+        if constexpr (Net::ACT == ACT_GELU) h[i] = gelu_approx2(pack2(a, b));
+        else h[i] = pack2(fmaxf(a, 0.0f), fmaxf(b, 0.0f));
+      }
+#pragma unroll
+      for (int o = 0; o < 3; ++o) {
+        const ulonglong2 w = reinterpret_cast<const ulonglong2*>(wo)[3 * (4 * c + q) + o];
+        s[o] = fma2(w.y, h[1], fma2(w.x, h[0], s[o]));
+      }
+    }
+  }
+#pragma unroll
+  for (int o = 0; o < 3; ++o) {
+    const float2 v = unpack2(s[o]);
+    rgb[o] = v.x + v.y;
   }
 }
 
@@ -274,7 +326,7 @@ __global__ void __launch_bounds__(Net::THREADS) __maxnreg__(Net::MAXREG)
       bool ok = true;
       for (int i = 0; i < tiles; ++i) {
 #pragma unroll
-        for (int k = 0; k < NL - 1; ++k) {
+        for (int k = 0; k < Net::MMA_LAYERS - 1; ++k) {
           ok = k == 0 ? wait(my_c0, c0_phase) : wait(my_c, c_phase);
           if (!ok) break;
           if (k == 0) c0_phase ^= 1u;
@@ -296,13 +348,19 @@ __global__ void __launch_bounds__(Net::THREADS) __maxnreg__(Net::MAXREG)
         if (!ok) break;
         c_phase ^= 1u;
         tc_fence_after();
-        uint32_t o[4];
-        tmem_ld4(t_base + reg, o);
-        tmem_ld_wait();
+        float rgb[3];
+        if constexpr (Net::OUT_FP32) {
+          output_layer<Net>(t_base + reg, reinterpret_cast<const float4*>(smem + Net::OFF_BO), rgb);
+        } else {
+          uint32_t o[4];
+          tmem_ld4(t_base + reg, o);
+          tmem_ld_wait();
+#pragma unroll
+          for (int c = 0; c < 3; ++c) rgb[c] = __uint_as_float(o[c]);
+        }
         tc_fence_before();
-        reg ^= N;  // the next tile's layer 0 went to the other region
-        write_rgb(p, out_img, b, y, x, __uint_as_float(o[0]) + bout[0], __uint_as_float(o[1]) + bout[1],
-                  __uint_as_float(o[2]) + bout[2]);
+        reg ^= N;  // the next tile's layer 0 goes to the other region
+        write_rgb(p, out_img, b, y, x, rgb[0] + bout[0], rgb[1] + bout[1], rgb[2] + bout[2]);
         y += 2;
         while (y >= p.H) {
           y -= p.H;
@@ -393,7 +451,7 @@ __global__ void __launch_bounds__(Net::THREADS) __maxnreg__(Net::MAXREG)
       const int tiles = (static_cast<int>(n * ((w >> 1) + 1) / kSets - s0) + 1 - par) / 2;
       bool ok = tiles > 0 && first_layer();
       for (int i = 0; i < tiles && ok; ++i) {
-        for (int k = 1; k < NL; ++k) {
+        for (int k = 1; k < Net::MMA_LAYERS; ++k) {
           const uint32_t ta = t_base + reg, d = t_base + (reg ^ N);
           reg ^= N;
           const bool out_layer = k == NL - 1;
