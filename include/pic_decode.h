@@ -255,6 +255,14 @@ int pic_decode_noalloc_check(void *stream);
  */
 int pic_decode_test_wait_fault(int withhold_arrival, unsigned spin_limit);
 
+/*
+ * Test hook (production code never calls it): how many times
+ * pic_decode_batch_noalloc has set up a kernel in this process, that is made
+ * CUDA calls other than the launch -- once per device and kernel, however
+ * many nets a kernel serves.
+ */
+int pic_decode_test_noalloc_setups(void);
+
 /* Frees the handle and its device state.  NULL is a no-op.  Synchronises the
  * device first, so that no kernel of this handle is still running. */
 void pic_decode_destroy(pic_decoder *h);

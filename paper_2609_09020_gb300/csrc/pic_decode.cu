@@ -603,7 +603,8 @@ namespace {
 
 constexpr int kStaticScratchInts = 64;  // 256 bytes; one call needs 1 word
 constexpr int kMaxStaticDevices = 64;
-constexpr int kNoallocKernelCache = 32;  // (device, kernel) pairs remembered
+constexpr int kNoallocKernels = 64;  // kernels remembered per device: more than the library has
+constexpr int kMaxResident = 16;     // CTAs of 128 threads (no decode kernel's has fewer) that an SM holds
 
 // What one device needs looked up once: its capabilities and the device
 // address of the static scratch (the array's name is only a host-side
@@ -614,20 +615,22 @@ struct NoallocDevice {
   int major, minor, sms, smem_optin;
   int* scratch;
 };
-// Per (device, kernel): the shared-memory attribute is set and the
-// occupancy and register count were read.
+// Per device and kernel: the shared-memory attribute is set and the
+// occupancy and register count were read.  A kernel that serves nets of any
+// size has its occupancy for all of them: fits[i] is the most dynamic shared
+// memory with which i + 1 CTAs are resident on an SM.
 struct NoallocKernel {
-  int dev;
   const void* fn;
-  int smem;  // (a generic kernel serves nets of several sizes)
-  int per_sm;
   bool regs_ok;
+  int resident;  // entries of fits
+  int fits[kMaxResident];
 };
 
 std::mutex g_noalloc_mutex;
 NoallocDevice g_noalloc_dev[kMaxStaticDevices];
-NoallocKernel g_noalloc_kern[kNoallocKernelCache];
-int g_noalloc_nkern = 0;
+NoallocKernel g_noalloc_kern[kMaxStaticDevices][kNoallocKernels];
+int g_noalloc_nkern[kMaxStaticDevices];
+int g_noalloc_setups = 0;  // (pic_decode_test_noalloc_setups)
 
 }  // namespace
 
@@ -660,33 +663,60 @@ int noalloc_device(int dev, NoallocDevice* out) {
   return PIC_OK;
 }
 
+// Resident CTAs of a kernel per SM with `smem` bytes of dynamic shared memory, -1 on failure.
+int resident_ctas(const KernelInfo& k, int smem) {
+  int n = 0;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k.fn, k.threads, smem) != cudaSuccess) {
+    cudaGetLastError();
+    return -1;
+  }
+  return n < kMaxResident ? n : kMaxResident;
+}
+
 // Occupancy of kernel `k` on `dev` (current), after setting its shared-memory
-// attribute; both done once per (device, kernel).
+// attribute; the CUDA calls for both are made once per (device, kernel).
 int noalloc_kernel(int dev, const KernelInfo& k, int* per_sm) {
   std::lock_guard<std::mutex> lock(g_noalloc_mutex);
-  for (int i = 0; i < g_noalloc_nkern; ++i)
-    if (g_noalloc_kern[i].dev == dev && g_noalloc_kern[i].fn == k.fn && g_noalloc_kern[i].smem == k.smem_bytes) {
-      if (!g_noalloc_kern[i].regs_ok) return PIC_ERR_UNSUPPORTED;
-      *per_sm = g_noalloc_kern[i].per_sm;
-      return PIC_OK;
+  NoallocKernel* const known = g_noalloc_kern[dev];
+  int& n_known = g_noalloc_nkern[dev];
+  NoallocKernel e{};
+  const NoallocKernel* found = nullptr;
+  for (int i = 0; i < n_known && !found; ++i)
+    if (known[i].fn == k.fn) found = &known[i];
+  if (!found) {
+    ++g_noalloc_setups;
+    e.fn = k.fn;
+    e.regs_ok = regs_match(k);
+    if (e.regs_ok) {
+      const int most = k.smem_attr ? k.smem_attr : k.smem_bytes;
+      if (cudaFuncSetAttribute(k.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, most) != cudaSuccess) {
+        cudaGetLastError();
+        return PIC_ERR_CUDA;
+      }
+      // fits[i], by bisection between what i + 1 CTAs are known to fit with and
+      // not (one query for a kernel of one size)
+      const int least = k.smem_attr ? 0 : k.smem_bytes;
+      e.resident = resident_ctas(k, least);
+      if (e.resident < 1) return PIC_ERR_UNSUPPORTED;
+      for (int i = 0; i < e.resident; ++i) {
+        int fit = least, over = most + 1;
+        while (k.smem_attr && over - fit > 1) {
+          const int mid = fit + (over - fit) / 2;
+          const int n = resident_ctas(k, mid);
+          if (n < 0) return PIC_ERR_UNSUPPORTED;
+          (n > i ? fit : over) = mid;
+        }
+        e.fits[i] = fit;
+      }
     }
-  NoallocKernel e{dev, k.fn, k.smem_bytes, 0, regs_match(k)};
-  if (e.regs_ok) {
-    if (cudaFuncSetAttribute(k.fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             k.smem_attr ? k.smem_attr : k.smem_bytes) != cudaSuccess) {
-      cudaGetLastError();
-      return PIC_ERR_CUDA;
-    }
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&e.per_sm, k.fn, k.threads, k.smem_bytes) !=
-            cudaSuccess ||
-        e.per_sm < 1) {
-      cudaGetLastError();
-      return PIC_ERR_UNSUPPORTED;
-    }
+    if (n_known < kNoallocKernels) known[n_known++] = e;
+    found = &e;
   }
-  if (g_noalloc_nkern < kNoallocKernelCache) g_noalloc_kern[g_noalloc_nkern++] = e;
-  if (!e.regs_ok) return PIC_ERR_UNSUPPORTED;
-  *per_sm = e.per_sm;
+  if (!found->regs_ok) return PIC_ERR_UNSUPPORTED;
+  int n = 0;
+  while (n < found->resident && k.smem_bytes <= found->fits[n]) ++n;
+  if (n < 1) return PIC_ERR_UNSUPPORTED;
+  *per_sm = n;
   return PIC_OK;
 }
 
@@ -757,6 +787,11 @@ extern "C" int pic_decode_batch_noalloc(const pic_arch* arch, int B, const int32
   DecodeParams p;
   fill_params(&h, p, B, latents, steps, weights, H, W, out_rgb);
   return launch(&h, p, static_cast<cudaStream_t>(stream));
+}
+
+extern "C" int pic_decode_test_noalloc_setups(void) {
+  std::lock_guard<std::mutex> lock(g_noalloc_mutex);
+  return g_noalloc_setups;
 }
 
 extern "C" int pic_decode_noalloc_check(void* stream) {

@@ -95,6 +95,8 @@ def load_library():
     lib.pic_decode_noalloc_check.restype = i
     lib.pic_decode_test_wait_fault.argtypes = [i, ctypes.c_uint]
     lib.pic_decode_test_wait_fault.restype = i
+    lib.pic_decode_test_noalloc_setups.argtypes = []
+    lib.pic_decode_test_noalloc_setups.restype = i
     lib.pic_decode_check.argtypes = [_P, _P]
     lib.pic_decode_check.restype = i
     lib.pic_decode_destroy.argtypes = [_P]
@@ -187,6 +189,10 @@ def pic_decode_batch_noalloc(arch: pic_arch, B, latents, steps, weights, H, W, o
 
 def pic_decode_noalloc_check(stream=None) -> int:
     return load_library().pic_decode_noalloc_check(stream)
+
+
+def pic_decode_test_noalloc_setups() -> int:
+    return load_library().pic_decode_test_noalloc_setups()
 
 
 def pic_decode_test_wait_fault(withhold_arrival: int, spin_limit: int) -> int:
