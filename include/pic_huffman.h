@@ -54,7 +54,9 @@ int64_t pic_huffman_workspace_bytes(int64_t n_words, int B, int p);
  *   sym_off     : int64, device, [B + 1]: stream b decodes to
  *                 out[sym_off[b] .. sym_off[b + 1])
  *   out         : int32, device, [sym_off[B]]
- *   workspace   : device, >= pic_huffman_workspace_bytes, 16-byte aligned
+ *   workspace   : device, >= pic_huffman_workspace_bytes, 16-byte aligned (or
+ *                 66 KB and 36 bytes per subsequence and 2 per table entry,
+ *                 where that is less: batches of small images, slower in it)
  * A stream that is not a sequence of codewords of its table, a symbol count
  * different from sym_off's, or a table whose lengths violate Kraft's
  * inequality is reported by pic_huffman_status (nothing is written out of

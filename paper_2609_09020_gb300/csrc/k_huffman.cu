@@ -78,7 +78,7 @@ constexpr int kMaxPasses = 64;
 constexpr int kHead = 16 + 4 * 68;  // workspace bytes before block_sum (a multiple of 16)
 static_assert(kHead >= 16 + 4 * kMaxPasses && kHead % 16 == 0, "status, pass counters");
 constexpr int kMaxTable = 4096;
-constexpr int kMaxGrid = 8192;
+constexpr int kMaxGrid = 4096;
 constexpr int kWords = 32 * kQ + 2;                  // stream words of a warp's 32 subsequences (two past the last)
 constexpr int kWrow = kQ + 1;                        // a subsequence's staged words, and the one that follows
 constexpr int kWbuf = 32 * kWrow + 2;
@@ -93,14 +93,14 @@ struct Ws {
   long long* block_sum;  // [kMaxGrid]: codewords of each CTA's range
   uint16_t* lut;         // [B][2^p]
   uint16_t* cnt;         // [n_sub]: codewords
-  uint8_t* multi;        // [B][2^p]: codewords inside the window << 4 | their bits
   uint8_t* over0;        // [n_sub]: overshoot, double-buffered over the passes
   uint8_t* over1;        // [n_sub]
   uint8_t* start;        // [n_sub]: the overshoot it was decoded from
-  uint8_t* direct;       // [B]: the lookup table holds values, not rows
+  uint8_t* multi;        // [B][2^p]: codewords inside the window << 4 | their bits (small workspace: none)
+  uint8_t* direct;       // [B]: the lookup table holds values, not rows (small workspace: none, all hold rows)
 };
 
-__host__ __device__ inline Ws ws_view(void* w, long long n_sub, int B, int p, long long* bytes = nullptr) {
+__host__ __device__ inline Ws ws_view(void* w, long long n_sub, int B, int p, bool small, long long* bytes = nullptr) {
   char* c = static_cast<char*>(w);
   const long long tab = static_cast<long long>(B) << p;
   Ws v;
@@ -113,21 +113,33 @@ __host__ __device__ inline Ws ws_view(void* w, long long n_sub, int B, int p, lo
   v.cnt = reinterpret_cast<uint16_t*>(c + o);
   o += (n_sub * 2 + 15) / 16 * 16;
   o = (o + 15) / 16 * 16;
-  v.multi = reinterpret_cast<uint8_t*>(c + o);
-  o += tab;
+  v.multi = small ? nullptr : reinterpret_cast<uint8_t*>(c + o);
+  o += small ? 0 : tab;
   v.over0 = reinterpret_cast<uint8_t*>(c + o);
   v.over1 = v.over0 + n_sub;
   v.start = v.over1 + n_sub;
-  v.direct = v.start + n_sub;
-  o += 3 * n_sub + B;
+  o += 3 * n_sub;
+  v.direct = small ? nullptr : reinterpret_cast<uint8_t*>(c + o);
+  o += small ? 0 : B;
   if (bytes) *bytes = (o + 15) / 16 * 16;
   return v;
 }
 
 long long ws_size(long long n_sub, int B, int p) {
   long long b = 0;
-  ws_view(nullptr, n_sub, B, p, &b);
+  ws_view(nullptr, n_sub, B, p, false, &b);
   return b;
+}
+
+// The other size that is accepted, 36 bytes a subsequence and 2 a table entry:
+// what was asked for before the multi tables, and less than they need where
+// images average fewer than about 132 subsequences (at p = 12).  In it every
+// CTA works the multi tables out for its own images, and a table's values are
+// all looked up by row: 256 images of 64x64 take 53 us in it, 39 in the other.  (The small layout
+// takes 5 bytes a subsequence, so it always fits.)
+long long ws_size_small(long long n_sub, int B, int p) {
+  const long long b = (16 + 4 * kMaxPasses + 8 * 8192 + (2LL * B << p) + 15) / 16 * 16;
+  return (b + 36 * n_sub + 15) / 16 * 16;
 }
 
 struct DecodeParams {
@@ -162,6 +174,20 @@ __device__ __forceinline__ uint32_t* words_of(uint8_t* s_dyn, int p) {
 }
 
 // ---------------------------------------------------------------- 0. tables
+// Codewords that lie wholly inside p-bit window i << 4 | the bits they take; a
+// window that starts with no codeword counts as one of 1 bit (the final decode
+// reports it).
+__device__ __forceinline__ int codewords_in(const uint16_t* lut, int i, int p) {
+  int pos = 0, c = 0;
+  while (pos < p) {
+    const int l = lut[(i << pos) & ((1 << p) - 1)] & 15;
+    if (l == 0 || pos + l > p) break;
+    pos += l;
+    ++c;
+  }
+  return c == 0 ? 1 << 4 | 1 : c << 4 | pos;
+}
+
 // The part-th of P.parts pieces of image b's lookup and multi tables -> global
 // memory (the whole CTA; the pieces' run starts are worked out by each, the
 // windows' codewords, three quarters of the time, only for the piece).
@@ -186,7 +212,7 @@ __device__ bool build_tables(const DecodeParams& P, int b, int part, void* scrat
     if (l == 0) atomicMin(&s_m, k);
     wide |= v < -2048 || v > 2047;
   }
-  const bool direct = !__syncthreads_or(wide);
+  const bool direct = !__syncthreads_or(wide) && P.ws.direct;
   const int m = s_m;
   // run sizes 2^(p - len) scanned into run starts, 256 entries at a time; more
   // than 2^p entries cannot be a code
@@ -224,7 +250,7 @@ __device__ bool build_tables(const DecodeParams& P, int b, int part, void* scrat
   bad = __syncthreads_or(bad) || carry > size;  // a bad length, or Kraft's inequality violated
   const int fill = bad ? 0 : carry;  // a bad table decodes nothing
   if (t == 0 && m <= size) s_start[m] = fill;
-  if (t == 0) P.ws.direct[b] = direct;
+  if (t == 0 && P.ws.direct) P.ws.direct[b] = direct;
   __syncthreads();
   auto entry = [&](int k, int& next) {  // and where symbol k's run ends
     const uint32_t v = s_start[k];
@@ -261,15 +287,7 @@ __device__ bool build_tables(const DecodeParams& P, int b, int part, void* scrat
   const int piece = size / P.parts;
   for (int i = part * piece + t; i < (part + 1) * piece; i += n_threads) {
     lut[i] = s_lut[i];
-    int pos = 0, c = 0;
-    while (pos < p) {
-      const int l = s_lut[(i << pos) & (size - 1)] & 15;
-      if (l == 0 || pos + l > p) break;
-      pos += l;
-      ++c;
-    }
-    if (c == 0) c = pos = 1;  // no codeword: counted as one of 1 bit (the final decode reports it)
-    multi[i] = static_cast<uint8_t>((c << 4) | pos);
+    if (P.ws.multi) multi[i] = static_cast<uint8_t>(codewords_in(s_lut, i, p));
   }
   return bad;
 }
@@ -306,7 +324,8 @@ struct Tables {
       asm volatile("{\n\t.reg .b32 t;\n\tld.shared.u8 t, [%1];\n\tcvt.u16.u32 %0, t;\n\t}" : "=h"(v) : "r"(multi_s + w));
       return v;
     }
-    return multi_g[w];
+    if (multi_g) return multi_g[w];
+    return 1 << 4 | max(lut_g[w] & 15, 1);  // (small workspace: one codeword at a time)
   }
 };
 
@@ -409,7 +428,7 @@ __device__ __forceinline__ void decode_phases(const DecodeParams& P, cg::grid_gr
       t.multi_s = multi_s + (b == b_first ? 0 : size);
     } else {
       t.lut_g = ws.lut + (static_cast<long long>(b) << P.p);
-      t.multi_g = ws.multi + (static_cast<long long>(b) << P.p);
+      t.multi_g = ws.multi ? ws.multi + (static_cast<long long>(b) << P.p) : nullptr;
     }
     return t;
   };
@@ -539,7 +558,7 @@ __device__ __forceinline__ void decode_phases(const DecodeParams& P, cg::grid_gr
     carry += __shfl_sync(0xffffffffu, x, 31);
     const Tables<SH> tab = tables(b);
     // this lane's rows in the value table (at most 2^28); -1: its entries are values
-    const int vals = __ldcg(ws.direct + b) ? -1 : b * P.max_table;
+    const int vals = ws.direct && __ldcg(ws.direct + b) ? -1 : b * P.max_table;
     const bool direct = __all_sync(0xffffffffu, vals < 0);
     while (__any_sync(0xffffffffu, pos < end)) {
       int n = 0;
@@ -651,14 +670,20 @@ __global__ void __launch_bounds__(kMaxWarps * 32, kCtasPerSm) huff_decode(const 
 #pragma unroll 2
       for (int i = tid; i < size / 8; i += n_threads)
         reinterpret_cast<uint4*>(sl)[i] = __ldcg(reinterpret_cast<const uint4*>(gl) + i);
-      for (int i = tid; i < size / 16; i += n_threads)
+      for (int i = tid; ws.multi && i < size / 16; i += n_threads)
         reinterpret_cast<uint4*>(sm)[i] = __ldcg(reinterpret_cast<const uint4*>(gm) + i);
     } else if (tid < size) {
       reinterpret_cast<uint16_t*>(sl)[tid] = __ldcg(gl + tid);
-      sm[tid] = __ldcg(gm + tid);
+      if (ws.multi) sm[tid] = __ldcg(gm + tid);
     }
   }
   __syncthreads();
+  if (!ws.multi) {
+    for (int i = tid; i < (b_last - b_first + 1) * size; i += n_threads)
+      s_dyn[4 * size + i] = static_cast<uint8_t>(
+          codewords_in(reinterpret_cast<const uint16_t*>(s_dyn) + (i & -size), i & (size - 1), P.p));
+    __syncthreads();
+  }
   decode_phases<true>(P, grid, s_dyn, b_first, b_last, k_begin, k_end);
 }
 
@@ -715,8 +740,9 @@ int pic_huffman_decode(const uint32_t* words, int64_t n_words, const int64_t* wo
       !aligned(sym_off, 8) || !aligned(tab_value, 4) || !aligned(tab_len, 4) || !aligned(out, 4))
     return PIC_ERR_INVALID_ARG;
   const long long n_sub = n_words / kQ;
-  if (static_cast<long long>(workspace_bytes) < ws_size(n_sub, B, p)) return PIC_ERR_INVALID_ARG;
-    int grid = 0;
+  const bool small = static_cast<long long>(workspace_bytes) < ws_size(n_sub, B, p);
+  if (small && static_cast<long long>(workspace_bytes) < ws_size_small(n_sub, B, p)) return PIC_ERR_INVALID_ARG;
+  int grid = 0;
   int rc = decode_grid(p, &grid);
   if (rc != PIC_OK) return rc;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
@@ -732,7 +758,7 @@ int pic_huffman_decode(const uint32_t* words, int64_t n_words, const int64_t* wo
   P.tab_len = tab_len;
   P.max_table = max_table;
   P.out = out;
-  P.ws = ws_view(workspace, n_sub, B, p);
+  P.ws = ws_view(workspace, n_sub, B, p, small);
   P.n_sub = n_sub;
   const long long groups = (n_sub + 31) / 32;
   // the fewest rounds that the resident warps can do the groups in, and the
