@@ -3,11 +3,13 @@
 //
 // Algorithm 1 expands each block from its end-of-block marker offsets, which
 // the paper finds beforehand by a stream compaction.  Here, with the stream
-// cut into 2048-symbol chunks and the chunks into one contiguous range per CTA:
-// 1. izpr_count: the eob markers of each range.
-// 2. izpr_expand: each CTA adds up the ranges before its own, which is its
-//    first block, and does the compaction and the expansion of its chunks
-//    together, chunk by chunk, as a segmented scan.  Each thread holds 16
+// cut into 2048-symbol chunks:
+// 1. izpr_count: the eob markers of each group of 4 chunks, and before each
+//    chunk within its group.
+// 2. izpr_expand: persistent CTAs do the compaction and the expansion
+//    together, chunk by chunk, as a segmented scan; a CTA takes every
+//    gridDim-th chunk and adds up the groups that it passes over, which gives
+//    it the chunk's first block.  Each thread holds 16
 //    consecutive symbols of the chunk in registers (loaded while the CTA
 //    expanded its previous chunk) and reduces them to (markers, positions
 //    covered since its last marker); warp 0 reads the 96 symbols before the
@@ -21,11 +23,17 @@
 // The stream is read twice; nothing else touches HBM but the coefficients and
 // offsets written.
 //
-// What bounds it: small streams, the launches -- two; there were four (a
-// memset of the status word, and a scan by one CTA of counts that chunks dealt
-// out round robin needed) -- and large ones, the instructions of the walks (66 for 32 symbols).
-// Measured, before and now: one 768x512 image (407 k symbols) 16.7 -> 12.1 us,
-// the 64-image batch (26 M symbols) 100 -> 91.6 us, one symbol 15.2 -> 9.5 us.
+// What bounds it: small streams, the launches -- two, where a memset of the
+// status word and a scan of the counts by one CTA made it four -- and large
+// ones, the instructions of the walks (66 for 32 symbols).
+// Measured, with four launches and now: one 768x512 image (407 k symbols) 16.7
+// -> 10.6 us, the 64-image batch (26 M symbols) 100 -> 96 us, one symbol 15.2 ->
+// 9.9 us.
+// Chunks differ in cost: one of 2,048 empty blocks writes 512 KB in 22 passes,
+// one of long blocks 10 KB in one.  Dealt out in turn, a flat stretch of the
+// stream is shared by all CTAs; in contiguous ranges, one per CTA, a few CTAs
+// get it whole.  64 images, the first 32 flat: 82 us in turn, 200 us in ranges,
+// which take 92 us on the even batch.
 #include <algorithm>
 #include <cstdint>
 
@@ -43,32 +51,31 @@ constexpr int kChunk = kThreads * kPerThread;  // symbols per compaction chunk
 
 enum : int { kBadBlock = 1, kBadCount = 2 };
 
-constexpr int kMaxGrid = 2048;  // ranges
+constexpr int kGroup = 4;  // chunks whose markers one CTA counts
+// CTAs of izpr_expand: its threads load at most three groups' counts each from
+// one of a CTA's chunks to the next
+constexpr int kMaxGrid = (3 * kThreads - 1) * kGroup;
 
-// Workspace: status word, and each range's markers.
+// Workspace: status word, each group's markers, and before each chunk those of
+// its group.  What callers provide is 5.5 bytes a chunk, as it was with groups
+// of 8 and their first blocks beside the counts: no less than these 5 take.
 struct Workspace {
   int* status;
-  int* count;
+  int* gcount;
+  int* local;
 };
 __host__ __device__ inline long long n_chunks_of(long long n) { return (n + kChunk - 1) / kChunk; }
-// What callers provide: 5.5 bytes a chunk, as the per-chunk counts took that
-// the ranges' replaced (32 + 4 x kMaxGrid bytes at most are used), so that the
-// same buffers stay accepted and refused.
+__host__ __device__ inline long long n_groups_of(long long n) { return (n_chunks_of(n) + kGroup - 1) / kGroup; }
 __host__ __device__ inline long long align16(long long b) { return (b + 15) / 16 * 16; }
 __host__ __device__ inline long long ws_bytes(long long n) {
-  const long long c = n_chunks_of(n), groups = (c + 7) / 8;
-  return 32 + align16(4 * groups) + align16(4 * c) + 8 * groups;
+  const long long c = n_chunks_of(n), eights = (c + 7) / 8;
+  return 32 + align16(4 * eights) + align16(4 * c) + 8 * eights;
 }
-__host__ __device__ inline Workspace ws_view(void* w) {
+__host__ __device__ inline Workspace ws_view(void* w, long long n) {
   char* p = static_cast<char*>(w);
-  return Workspace{reinterpret_cast<int*>(p), reinterpret_cast<int*>(p + 32)};
+  return Workspace{reinterpret_cast<int*>(p), reinterpret_cast<int*>(p + 32),
+                   reinterpret_cast<int*>(p + 32 + align16(4 * n_groups_of(n)))};
 }
-// CTA i's chunks: `per` each, one more for the first `more` CTAs.
-struct Ranges {
-  long long per;
-  int more;
-  __device__ __forceinline__ long long first(int cta) const { return cta * per + min(cta, more); }
-};
 
 // Zigzag order of an 8x8 block (raster index of the k-th zigzag position):
 // anti-diagonal d = row + col, row falling for even d, rising for odd d.
@@ -109,48 +116,58 @@ __device__ __forceinline__ void load16(const int32_t* __restrict__ sym, long lon
   }
 }
 
-// The markers of each range.  What bounds it is DRAM, with 16-byte loads
-// coalesced over the CTA and kAhead of them in flight.
-constexpr int kCountThreads = 256;
+// The markers of group blockIdx.x, and before each of its chunks.  What bounds
+// it is DRAM for large streams (6 TB/s) and one load's latency for small ones:
+// thread t loads symbols 4t .. 4t + 3 of all four chunks at once (groups of 8:
+// the same, and one image 5.0 instead of 3.4 us).
+constexpr int kCountThreads = kChunk / 4;
 __global__ void __launch_bounds__(kCountThreads) izpr_count(const int32_t* __restrict__ sym, long long n, int32_t eob,
-                                                            Ranges ranges, Workspace ws) {
-  __shared__ int s_warp[kCountThreads / 32];
-  constexpr int kStep = 4 * kCountThreads, kAhead = 8;
-  const int t = threadIdx.x;
+                                                            long long n_chunks, Workspace ws) {
+  constexpr int kWarps = kCountThreads / 32;
+  __shared__ unsigned s_cnt[kWarps];
+  const int t = threadIdx.x, lane = t & 31;
+  const long long c0 = static_cast<long long>(blockIdx.x) * kGroup, i0 = c0 * kChunk + 4 * t;
   const bool vec = (reinterpret_cast<uintptr_t>(sym) & 15u) == 0;
-  const long long end = min(ranges.first(blockIdx.x + 1) * kChunk, n);
-  long long i = ranges.first(blockIdx.x) * kChunk + 4 * t;
-  int cnt = 0;
-  for (; vec && i + kStep * (kAhead - 1) + 3 < end; i += kStep * kAhead) {
-    int4 v[kAhead];
+  static_assert(kGroup == 4 && kWarps <= 32, "a byte per chunk, a lane per warp");
+  unsigned cnt = 0u;  // a byte per chunk: at most 4 a thread, 128 a warp
+  if (vec && (c0 + kGroup) * kChunk <= n) {
+    int4 v[kGroup];
 #pragma unroll
-    for (int j = 0; j < kAhead; ++j) v[j] = __ldg(reinterpret_cast<const int4*>(sym + i) + kCountThreads * j);
+    for (int k = 0; k < kGroup; ++k) v[k] = __ldg(reinterpret_cast<const int4*>(sym + i0 + k * kChunk));
 #pragma unroll
-    for (int j = 0; j < kAhead; ++j) cnt += (v[j].x == eob) + (v[j].y == eob) + (v[j].z == eob) + (v[j].w == eob);
-  }
-  for (; i < end; i += kStep) {
-    if (vec && i + 3 < end) {
-      const int4 v = __ldg(reinterpret_cast<const int4*>(sym + i));
-      cnt += (v.x == eob) + (v.y == eob) + (v.z == eob) + (v.w == eob);
-    } else {
+    for (int k = 0; k < kGroup; ++k)
+      cnt += static_cast<unsigned>((v[k].x == eob) + (v[k].y == eob) + (v[k].z == eob) + (v[k].w == eob)) << 8 * k;
+  } else {
 #pragma unroll
-      for (int u = 0; u < 4; ++u) cnt += i + u < end && __ldg(sym + i + u) == eob;
+    for (int k = 0; k < kGroup; ++k) {
+      const long long i = i0 + k * kChunk;
+#pragma unroll
+      for (int u = 0; u < 4; ++u) cnt += static_cast<unsigned>(i + u < n && __ldg(sym + i + u) == eob) << 8 * k;
     }
   }
   cnt = __reduce_add_sync(0xffffffffu, cnt);
-  if (t % 32 == 0) s_warp[t / 32] = cnt;
+  if (lane == 0) s_cnt[t / 32] = cnt;
   __syncthreads();
-  if (t == 0) {
-    for (int w = 1; w < kCountThreads / 32; ++w) cnt += s_warp[w];
-    ws.count[blockIdx.x] = cnt;
-    if (blockIdx.x == 0) *ws.status = 0;
+  if (t >= 32) return;
+  const unsigned x = lane < kWarps ? s_cnt[lane] : 0u;
+  const unsigned even = __reduce_add_sync(0xffffffffu, x & 0x00FF00FFu), odd = __reduce_add_sync(0xffffffffu, x >> 8 & 0x00FF00FFu);
+  if (lane == 0) {
+    const int m[4] = {static_cast<int>(even & 0xFFFF), static_cast<int>(odd & 0xFFFF), static_cast<int>(even >> 16), static_cast<int>(odd >> 16)};
+    int run = 0;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      if (c0 + k < n_chunks) ws.local[c0 + k] = run;
+      run += m[k];
+    }
+    ws.gcount[blockIdx.x] = run;
   }
+  if (t == 0 && blockIdx.x == 0) *ws.status = 0;
 }
 
 // Compaction and expansion in one pass over the stream, as a segmented scan.
 // A block holds at most 64 symbols before its marker, so the marker that
 // precedes a chunk's first block lies within the kHalo symbols before the
-// chunk (or the block is malformed).  For each chunk of the CTA's range:
+// chunk (or the block is malformed).  CTAs take chunks c, c + grid, ...; for each:
 //  - every thread holds 16 consecutive symbols of the chunk in registers
 //    (loaded while the CTA worked on its previous chunk) and reduces them to
 //    (markers, positions covered since its last marker);
@@ -186,8 +203,8 @@ __device__ __forceinline__ Seg seg_cat(Seg a, Seg b) { return Seg{a.m + b.m, b.m
 
 __global__ void __launch_bounds__(kThreads, 8) izpr_expand(const int32_t* __restrict__ sym,
                                                         long long n, int32_t eob,
-                                                        Ranges ranges, const int* __restrict__ count,
-                                                        long long n_blocks,
+                                                        long long n_chunks, const int* __restrict__ gcount,
+                                                        const int* __restrict__ local, long long n_blocks,
                                                         int32_t* __restrict__ coeffs,
                                                         int64_t* __restrict__ offsets, int* status) {
   extern __shared__ __align__(16) unsigned char smem[];
@@ -197,7 +214,6 @@ __global__ void __launch_bounds__(kThreads, 8) izpr_expand(const int32_t* __rest
   int* s_carry = reinterpret_cast<int*>(s_zz + 64);
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
   constexpr int kWarps = kThreads / 32;
-  const long long c_begin = ranges.first(blockIdx.x), c_end = ranges.first(blockIdx.x + 1);
   if (t < 64) s_zz[t] = static_cast<unsigned char>(make_zigzag().v[t]);
   if (blockIdx.x == 0 && t == 0) {
     if (__ldg(sym + n - 1) != eob) atomicOr(status, kBadCount);  // symbols after the last marker
@@ -218,49 +234,51 @@ __global__ void __launch_bounds__(kThreads, 8) izpr_expand(const int32_t* __rest
     for (int u = 0; u < 3; ++u) h[u] = (warp != 0 || hi + u < 0) ? eob : __ldg(sym + hi + u);
   };
 
-  // the next chunk's symbols and halo, loaded one chunk ahead
-  int cur[16], hcur[3];
-  load16(sym, n, c_begin * kChunk + 16 * t, vec, fill, cur);
-  load_halo(c_begin, hcur);
-  // the blocks of the ranges before this one; of all ranges
-  long long gb0 = 0;
-  {
-    long long before = 0, all = 0;
-    for (int i = t; i < static_cast<int>(gridDim.x); i += kThreads) {
-      const int v = count[i];
-      before += i < static_cast<int>(blockIdx.x) ? v : 0;
-      all += v;
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      before += __shfl_xor_sync(0xffffffffu, before, o);
-      all += __shfl_xor_sync(0xffffffffu, all, o);
-    }
-    long long* s_sum = reinterpret_cast<long long*>(s_scan);
-    if (lane == 0) {
-      s_sum[2 * warp] = before;
-      s_sum[2 * warp + 1] = all;
-    }
-    __syncthreads();
-    all = 0;
-#pragma unroll
-    for (int w = 0; w < kWarps; ++w) {
-      gb0 += s_sum[2 * w];
-      all += s_sum[2 * w + 1];
-    }
-    if (blockIdx.x == 0 && t == 0 && all != n_blocks) atomicOr(status, kBadCount);
-    __syncthreads();
-  }
-  for (long long c = c_begin; c < c_end; ++c) {
+  // the blocks before group g: the counts of the groups passed over, up to three a thread
+  int* const s_sum = s_scan + 2 * kWarps;
+  int passed[3];
+  auto load_passed = [&](long long g, long long g_next) {
+    const int* const from = gcount + g + t;
+    const int left = static_cast<int>(g_next - g) - t;
+    passed[0] = left > 0 ? __ldg(from) : 0;
+    passed[1] = left > kThreads ? __ldg(from + kThreads) : 0;
+    passed[2] = left > 2 * kThreads ? __ldg(from + 2 * kThreads) : 0;
+  };
+  auto put_passed = [&]() {
+    const int sum = __reduce_add_sync(0xffffffffu, passed[0] + passed[1] + passed[2]);
+    if (lane == 0) s_sum[warp] = sum;
+  };
+  long long group_base = 0;
+  auto add_passed = [&]() {
+    static_assert(kWarps == 4, "one word per warp");
+    const int4 q = *reinterpret_cast<const int4*>(s_sum);
+    group_base += q.x + q.y + q.z + q.w;
+  };
+
+  // the next chunk's symbols, halo and first block, loaded one chunk ahead
+  int cur[16], hcur[3], lcur = 0;
+  const long long grid = gridDim.x;
+  load16(sym, n, blockIdx.x * static_cast<long long>(kChunk) + 16 * t, vec, fill, cur);
+  load_halo(blockIdx.x, hcur);
+  lcur = __ldg(local + blockIdx.x);
+  load_passed(0, blockIdx.x / kGroup);
+  put_passed();
+  __syncthreads();
+  add_passed();
+  for (long long c = blockIdx.x; c < n_chunks; c += grid) {
+    const long long gb0 = group_base + lcur;
     const long long c0 = c * kChunk;
     int x16[16], h[3];
 #pragma unroll
     for (int i = 0; i < 16; ++i) x16[i] = cur[i];
 #pragma unroll
     for (int u = 0; u < 3; ++u) h[u] = hcur[u];
-    if (c + 1 < c_end) {  // next chunk, in flight meanwhile
-      load16(sym, n, (c + 1) * kChunk + 16 * t, vec, fill, cur);
-      load_halo(c + 1, hcur);
+    const bool more = c + grid < n_chunks;
+    if (more) {  // next chunk, in flight meanwhile
+      load16(sym, n, (c + grid) * kChunk + 16 * t, vec, fill, cur);
+      load_halo(c + grid, hcur);
+      lcur = __ldg(local + c + grid);
+      load_passed(c / kGroup, (c + grid) / kGroup);
     }
 
     // this thread's markers (bit i: symbol i) and positions since its last one
@@ -385,8 +403,10 @@ __global__ void __launch_bounds__(kThreads, 8) izpr_expand(const int32_t* __rest
       __syncthreads();  // the slots are clear again
     }
     if (bad) atomicOr(status, kBadBlock);
-    gb0 += tot;
+    if (c + 1 == n_chunks && t == 0 && gb0 + tot != n_blocks) atomicOr(status, kBadCount);
+    if (more) put_passed();
     __syncthreads();  // the scan scratch and the halo carry are free again
+    if (more) add_passed();
   }
 }
 
@@ -442,16 +462,15 @@ int pic_izpr_decode(const int32_t* symbols, int64_t n_symbols, int32_t eob, int6
     return PIC_ERR_INVALID_ARG;
   if (eob < INT32_MIN + 17) return PIC_ERR_INVALID_ARG;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  const Workspace ws = ws_view(workspace);
+  const Workspace ws = ws_view(workspace, n_symbols);
   const long long chunks = n_chunks_of(n_symbols);
   if (chunks > 0) {
     int grid = 0;
     if (expand_grid(&grid) != PIC_OK) return PIC_ERR_CUDA;
-    const int g = static_cast<int>(std::min<long long>(chunks, grid));
-    const Ranges ranges{chunks / g, static_cast<int>(chunks % g)};
-    izpr_count<<<g, kCountThreads, 0, s>>>(symbols, n_symbols, eob, ranges, ws);
-    izpr_expand<<<g, kThreads, kExpandSmem, s>>>(symbols, n_symbols, eob, ranges, ws.count, n_blocks, coeffs, offsets,
-                                                 ws.status);
+    izpr_count<<<static_cast<unsigned>(n_groups_of(n_symbols)), kCountThreads, 0, s>>>(symbols, n_symbols, eob, chunks,
+                                                                                     ws);
+    izpr_expand<<<static_cast<unsigned>(std::min<long long>(chunks, grid)), kThreads, kExpandSmem, s>>>(
+        symbols, n_symbols, eob, chunks, ws.gcount, ws.local, n_blocks, coeffs, offsets, ws.status);
   } else {
     izpr_flag<<<1, 1, 0, s>>>(ws.status, n_blocks > 0 ? kBadCount : 0);  // no symbols, hence no markers
   }
