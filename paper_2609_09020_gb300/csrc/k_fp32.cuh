@@ -607,8 +607,17 @@ __device__ __forceinline__ void any_layer(float* __restrict__ X, const float* __
 
 constexpr int kAnyBatch = 4;
 
+// CTAs per SM that the registers allow.  Nets up to 16 wide have the fewest
+// FMAs between barriers and gain most from more of them: 7 instead of 5,
+// 6-8-8-3, 16 images of 64x64 (1,024 tiles, one round on 152 SMs) 12.4 -> 10.5
+// us, one of 768x512 20.7 -> 18.7 us; 8 spill (4-16-16-16-16-16-3, one 768x512
+// image 43 -> 45 us).
+__host__ __device__ constexpr int any_min_ctas(int max_t2) {
+  return max_t2 <= 2 ? 7 : max_t2 <= 5 ? 5 : max_t2 <= 8 ? 4 : 2;
+}
+
 template <int MAXT2, bool FL>
-__global__ void __launch_bounds__(kThreads, MAXT2 <= 5 ? 5 : (MAXT2 <= 8 ? 4 : 2))
+__global__ void __launch_bounds__(kThreads, any_min_ctas(MAXT2))
     fp32_any_kernel(const DecodeParams p) {
   extern __shared__ __align__(16) float smem[];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
