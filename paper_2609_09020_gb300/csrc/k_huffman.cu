@@ -51,6 +51,7 @@
 // subsequences an image): 1 image 54.3 -> 24.8 us, 24 images 100.2 -> 45.4 us,
 // 64 images 163 -> 96.5 us; 256 images of 64x64 108 -> 38.4 us.
 #include <algorithm>
+#include <atomic>
 #include <cstdint>
 
 #include <cooperative_groups.h>
@@ -704,7 +705,7 @@ bool aligned(const void* p, uintptr_t a) { return (reinterpret_cast<uintptr_t>(p
 // lookup tables each (the cooperative grid), per device and precision.
 int decode_grid(int p, int* grid) {
   constexpr int kMaxDev = 64;
-  static int cached[kMaxDev][PIC_HUFF_MAX_PRECISION + 1];
+  static std::atomic<int> cached[kMaxDev][PIC_HUFF_MAX_PRECISION + 1];  // (first calls may come from several threads)
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDev) {
     cudaGetLastError();

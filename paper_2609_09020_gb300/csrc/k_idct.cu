@@ -29,6 +29,7 @@
 // X[1, 3, 5, 7] -- 36 operations instead of 64 multiply-adds.  The patch
 // slot is padded to 72 floats so the column accesses of pass 2 hit 32
 // distinct banks.
+#include <atomic>
 #include <cstdint>
 
 #include <cuda_runtime.h>
@@ -185,7 +186,7 @@ bool sizes_ok(int H, int W, int L, int C) {
 // Resident CTAs of the kernel on the current device, set up once per device.
 int idct_grid(int* grid) {
   constexpr int kMaxDev = 64;
-  static int cached[kMaxDev];
+  static std::atomic<int> cached[kMaxDev];  // (first calls may come from several threads at once)
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDev) {
     cudaGetLastError();

@@ -35,6 +35,7 @@
 // get it whole.  64 images, the first 32 flat: 82 us in turn, 200 us in ranges,
 // which take 92 us on the even batch.
 #include <algorithm>
+#include <atomic>
 #include <cstdint>
 
 #include <cuda_runtime.h>
@@ -417,7 +418,7 @@ bool aligned(const void* p, uintptr_t a) { return (reinterpret_cast<uintptr_t>(p
 // Resident CTAs of izpr_expand on the current device, set up once per device.
 int expand_grid(int* grid) {
   constexpr int kMaxDev = 64;
-  static int cached[kMaxDev];
+  static std::atomic<int> cached[kMaxDev];  // (first calls may come from several threads at once)
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDev) {
     cudaGetLastError();
