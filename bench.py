@@ -79,27 +79,18 @@ GELU_FP32_OPS = 4 + 5 + 4
 def march_tensor_macs_per_px(wl: wk.Workload) -> int:
     """MACs the tensor cores execute per pixel in the row-marching kernels (the
     ones staging "auto" picks): layer 0 (K = the hi and lo features and the
-    constant 1, round16), hidden layers and the output layer with the hi and lo
-    halves of K.  Nets wider than 40 run on N = 64 tiles, each bias that is no
-    column of layer 0 as one K = 16 step and the output layer as N = 16;
-    narrower ones at their own width, biases free, the output layer as N = 8."""
+    constant 1, round16), hidden layers and the output layer (where it is not in
+    fp32 on the CUDA cores) with the hi and lo halves of K.  Nets wider than 40
+    run on N = 64 tiles, each bias that is no column of layer 0 as one K = 16
+    step and the output layer as N = 16; narrower ones at their own width,
+    biases free, the output layer as N = 8."""
     d0, width = wl.dims[0], max(wl.dims[1:-1])
     k1 = (4 * ((d0 + 1) // 2) + 15) // 16 * 16
     bias_column = d0 % 2 == 1 or 4 * ((d0 + 1) // 2) < k1
     n, bias, out = (64, 16, 16) if width > 40 else ((width + 7) // 8 * 8, 0, 8)
     mac = (k1 + (0 if bias_column else bias)) * n
     mac += (len(wl.dims) - 3) * (2 * n + bias) * n
-    return mac + 2 * n * out
-
-
-def march_alu_ops_per_px(wl: wk.Workload, precision: str) -> int:
-    """Activation-inclusive CUDA-core work per pixel (FP32-pipe operations):
-    every hidden activation (GELU at GELU_OPS; ReLU is folded into a
-    conversion), plus on the tensor path the hi/lo split of every hidden value
-    (2 per value), plus on the fp32 path every MLP MAC."""
-    hidden = sum(wl.dims[1:-1])
-    ops = (GELU_OPS if wl.act == "gelu" else 0) * hidden
-    return ops + (2 * hidden if precision == "fp16_tc" else wl.macs_per_pixel)
+    return mac + (2 * n * out if tc_output_on_tensor_cores(wl) else 0)
 
 
 def executed_tensor_macs_per_px(wl: wk.Workload) -> int:
@@ -119,21 +110,21 @@ def executed_tensor_macs_per_px(wl: wk.Workload) -> int:
 
 
 def tc_output_on_tensor_cores(wl: wk.Workload) -> bool:
-    """The per-tile kernels run the output layer as an MMA only for wide, shallow
-    nets (padded width > 32 and fewer than 4 layers); else on the CUDA cores."""
+    """The tensor-core kernels run the output layer as an MMA only for wide, shallow
+    nets (width > 32 and fewer than 4 layers); else on the CUDA cores."""
     n_pad = (max(wl.dims[1:-1]) + 15) // 16 * 16
     return n_pad > 32 and len(wl.dims) - 1 < 4
 
 
-def alu_ops_per_px(wl: wk.Workload, precision: str) -> int:
-    """Activation-inclusive CUDA-core work per pixel (FP32-pipe operations) of
-    the per-tile kernels with the rational GELU, for comparison with older
-    figures: every hidden activation (GELU at GELU_FP32_OPS; ReLU is folded into
-    a conversion), plus on the tensor path the hi/lo split of every hidden value
-    that feeds an MMA (2 per value) and the output layer where it runs on the
-    CUDA cores (one FMA per weight), plus on the fp32 path every MLP MAC."""
+def alu_ops_per_px(wl: wk.Workload, precision: str, gelu_ops: int = GELU_FP32_OPS) -> int:
+    """Activation-inclusive CUDA-core work per pixel (FP32-pipe operations):
+    every hidden activation (GELU at gelu_ops, GELU_OPS in the kernels; ReLU is
+    folded into a conversion or runs beside the FP32 pipe), plus on the tensor
+    path the hi/lo split of every hidden value that feeds an MMA (2 per value)
+    and the output layer where it runs on the CUDA cores (one FMA per weight),
+    plus on the fp32 path every MLP MAC."""
     hidden = list(wl.dims[1:-1])
-    act = GELU_FP32_OPS if wl.act == "gelu" else 0
+    act = gelu_ops if wl.act == "gelu" else 0
     ops = act * sum(hidden)
     if precision == "fp16_tc":
         if tc_output_on_tensor_cores(wl):
@@ -146,8 +137,9 @@ def alu_ops_per_px(wl: wk.Workload, precision: str) -> int:
 
 
 def roofline_for(wl: wk.Workload, precision: str, B: int, ms: float, peaks: dict,
-                 fp32_tflops: float, fp32_src: str) -> dict:
-    """The roofline of one decode launch of B images that took ms: the binding
+                 fp32_tflops: float, fp32_src: str, staging: str = "auto") -> dict:
+    """The roofline of one decode launch of B images that took ms with the kernel
+    that staging picks: the binding
     of (unpadded MLP FLOPs at the path's pipe peak, algorithmic bytes at the
     HBM peak), and beside it the activation-inclusive ALU bound."""
     flops, nbytes = algorithmic(wl, B)
@@ -169,13 +161,14 @@ def roofline_for(wl: wk.Workload, precision: str, B: int, ms: float, peaks: dict
     roof["frac"] = roof["achieved"] / roof["peak"]
     roof["algorithmic_flops_per_launch"] = flops
     if precision == "fp16_tc":
-        roof["executed_tensor_flops_per_launch"] = 2.0 * march_tensor_macs_per_px(wl) * px
+        macs = march_tensor_macs_per_px if staging == "auto" else executed_tensor_macs_per_px
+        roof["executed_tensor_flops_per_launch"] = 2.0 * macs(wl) * px
     roof["algorithmic_bytes_per_launch"] = nbytes
     roof["binding_time_us"] = max(t_pipe, t_hbm) * 1e6
     roof["avg_launch_us"] = ms * 1e3
     # activation-inclusive ALU bound (FP32 pipe at the measured FMA rate;
     # one operation = one lane-op, half an FMA's two FLOPs)
-    ops = march_alu_ops_per_px(wl, precision)
+    ops = alu_ops_per_px(wl, precision, GELU_OPS)
     t_alu = ops * px / (fp32_tflops * 1e12 / 2)
     t_bind = max(t_pipe, t_hbm, t_alu)
     roof["alu_bound"] = {"ops_per_px": ops,
@@ -188,15 +181,26 @@ def roofline_for(wl: wk.Workload, precision: str, B: int, ms: float, peaks: dict
 KERNEL_SOURCES = {
     "idct": ["k_idct.cu"],
     "izpr": ["k_izpr.cu"],
-    "tc": ["k_tcmarch.cuh", "march.cuh", "tc_ptx.cuh", "pic_common.cuh", "pic_gelu.cuh", "pic_kernels.h"],
+    "tc_march": ["k_tcmarch.cuh", "march.cuh", "tc_ptx.cuh", "pic_common.cuh", "pic_gelu.cuh", "pic_kernels.h"],
+    "tc_strip": ["k_strip.cuh", "march.cuh", "tc_ptx.cuh", "pic_common.cuh", "pic_gelu.cuh", "pic_kernels.h"],
+    "tc_tile": ["k_tc.cuh", "tc_ptx.cuh", "pic_common.cuh", "pic_gelu.cuh", "pic_kernels.h"],
     "fp32": ["k_fp32.cuh", "pic_common.cuh", "pic_gelu.cuh", "pic_kernels.h"],
 }
 
 
+def kernel_sources(kernel_name: str):
+    """The source files that a decode kernel, by its name, is compiled from."""
+    if kernel_name.startswith("tc"):
+        if kernel_name.endswith(("_tile", "_tma", "_lo8")):
+            return KERNEL_SOURCES["tc_tile"]
+        dims = [int(d) for d in kernel_name.split("_")[1].split("x")]
+        return KERNEL_SOURCES["tc_strip" if max(dims[1:-1]) <= 40 else "tc_march"]
+    return KERNEL_SOURCES[next((k for k in ("idct", "izpr") if kernel_name.startswith(k)), "fp32")]
+
+
 def kernel_source_hash(kernel_name: str) -> str:
     """Hash of the source files a decode kernel is compiled from."""
-    key = next((k for k in ("tc", "idct", "izpr") if kernel_name.startswith(k)), "fp32")
-    files = KERNEL_SOURCES[key]
+    files = kernel_sources(kernel_name)
     h = hashlib.sha256()
     csrc = os.path.join(ROOT, "paper_2609_09020_gb300", "csrc")
     for fn in files:
@@ -926,8 +930,8 @@ def fp32_peak(pic, dev):
 
 
 PER_CONFIG = ["c1", "c2", "c3", "c4", "c5"]
-# extra tensor-path rows with the latent staging the library's default does
-# not pick for that architecture (TMA boxes vs per-thread copies)
+# extra tensor-path rows with the per-tile kernels' TMA staging, which the
+# library's default (the row-marching kernels) does not pick
 PER_CONFIG_STAGING = {"c5": "tma", "c3": "tma", "c4": "tma"}
 
 
@@ -969,7 +973,7 @@ def per_config_rows(pic, dev, stream, peaks, fp32_tf, fp32_src, reps=None):
                 times.append(e0.elapsed_time(e1))
             dec.check(stream)
             ms = float(np.median(times))
-            roof = roofline_for(wl, precision, B, ms, peaks, fp32_tf, fp32_src)
+            roof = roofline_for(wl, precision, B, ms, peaks, fp32_tf, fp32_src, staging)
             rows.append({"workload": name, "precision": precision, "staging": staging,
                          "kernel": dec.kernel_name,
                          "images": B, "ms": ms, "ms_p10": float(np.percentile(times, 10)),
