@@ -65,7 +65,11 @@ typedef enum {
     /* fp16 weights; the MLP runs on the tensor cores with fp16 operands and
      * fp32 accumulation.  Every activation operand (features and hidden
      * values) is split into two fp16 terms hi + lo, so the products carry
-     * about 22 significant bits; the weights are used exactly as given. */
+     * about 22 significant bits (fewer below 2^-3, where lo's absolute step of
+     * 2^-24 shows) and the operand must stay below 131,008 in magnitude; the
+     * weights are used exactly as given.  The last hidden values are no operand
+     * of nets at most 32 wide or with four layers or more: their output layer
+     * runs in fp32. */
     PIC_PREC_FP16_TC = 1,
     /* fp16 weights; tensor cores as PIC_PREC_FP16_TC, with the lo term of
      * every hidden operand in fp8 (e4m3) against an e4m3 copy of the

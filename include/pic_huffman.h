@@ -61,8 +61,12 @@ int64_t pic_huffman_workspace_bytes(int64_t n_words, int B, int p);
  * different from sym_off's, or a table whose lengths violate Kraft's
  * inequality is reported by pic_huffman_status (nothing is written out of
  * bounds; the output is then unspecified), as is a stream whose parallel
- * decodings do not synchronise within 64 passes (never seen on Huffman codes;
- * the result is then unspecified too).
+ * decodings do not synchronise within 64 passes (the result is then unspecified
+ * too).  A pass sets one more 256-bit piece of a stream right for certain, and
+ * codes of different lengths fall into step within a few codewords; but where
+ * all codewords, or nearly all, have one length that does not divide 256, a
+ * decoding that starts inside one stays out of step, so such a stream is
+ * refused if it is longer than about 64 pieces.
  * Errors: PIC_ERR_INVALID_ARG, PIC_ERR_UNSUPPORTED (no cooperative launch on
  * this device), PIC_ERR_CUDA.
  */

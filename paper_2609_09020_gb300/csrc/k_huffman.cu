@@ -4,8 +4,8 @@
 //
 // One cooperative launch (every CTA resident, grid-wide barriers between the
 // phases):
-//    0. tables: the CTAs expand the stored tables, up to kMaxParts CTAs to an
-//       image.  A table -- values and lengths in canonical order -- is the
+//    0. tables (for more images than CTAs by a launch of their own): the CTAs
+//       expand the stored tables, up to kMaxParts CTAs to an image.  A table -- values and lengths in canonical order -- is the
 //       run-length code of the 2^p-entry lookup table: symbol k covers
 //       2^(p - len_k) consecutive entries.  Expanding the runs gives the table,
 //       so one lookup of the next p bits decodes a symbol.  A 16-bit entry is
@@ -22,10 +22,11 @@
 //    b. synchronisation passes: a subsequence whose predecessor's overshoot
 //       differs from the one it was decoded with is decoded again from there
 //       (in the first pass every one is, and counts its codewords).
-//       Prefix codes resynchronise within a few codewords, so a pass seldom
-//       changes an overshoot, and the passes end with the first that changes
-//       none (usually the first); pass i has made subsequence i exact, and
-//       after 64 passes without convergence the status word says so.  Each
+//       Codes of different lengths resynchronise within a few codewords, so a
+//       pass seldom changes an overshoot, and the passes end with the first that
+//       changes none (usually the first); pass i has made subsequence i exact,
+//       and after 64 passes without convergence (codewords of one length that
+//       does not divide 256) the status word says so.  Each
 //       pass also leaves the CTAs' codeword totals, from which
 //    c. every CTA takes its output position (the total must equal the symbol
 //       offsets');
@@ -48,7 +49,8 @@
 // against the lookup's 30), the tables came from a launch of their own and a
 // memset, CTA barriers held every warp to the slowest, and the passes kept 36
 // bytes a subsequence instead of 5.  Measured, before and now (768x512, 6,800
-// subsequences an image): 1 image 54.3 -> 24.8 us, 24 images 100.2 -> 45.4 us,
+// subsequences an image, the streams of perf/cases.py's distribution; the 24 of
+// another seed, with a few more, 48 us): 1 image 54.3 -> 24.8 us, 24 images 100.2 -> 45.4 us,
 // 64 images 163 -> 96.5 us; 256 images of 64x64 108 -> 38.4 us.
 #include <algorithm>
 #include <atomic>
@@ -69,7 +71,8 @@ constexpr int kS = 32 * kQ;                     // bits per subsequence
 // Warps of a CTA: 8, or 9 where that saves a round of groups (24 images of
 // 768x512, 5,129 groups on 152 SMs: 45.4 us in one round, 64 in two).  Nine
 // warps of 56 registers on each of four CTAs fill an SM; ten, at 48
-// registers, spill (69 us).  Fewer than 8 make the tables too slowly (one
+// registers, spill (69 us).  Held to eight warps and 64 registers, 1 and 64
+// images take the same time within 1 %, and 24 images 55.6 us.  Fewer than 8 make the tables too slowly (one
 // image: 33 us with 2, 26.9 with 4, 25.9 with 8).
 constexpr int kMaxWarps = 9;
 constexpr int kMinWarps = 8;
@@ -151,7 +154,7 @@ struct DecodeParams {
   int B;
   int p;
   const long long* sym_off;
-  const int32_t* tab_value;  // [B][max_table]: a table entry's low 12 bits index its row
+  const int32_t* tab_value;  // [B][max_table]: a row entry's high 12 bits index it
   const int32_t* tab_len;    // [B][max_table]
   int max_table;
   int32_t* out;

@@ -12,11 +12,11 @@
 // tcgen05's rate (8.2 cycles per m16n8k16 and sub-partition) and each one
 // takes about 6 cycles of the FMA pipe besides, so its share grows with the
 // square of the width; up to 40 it pays.  64 images of 768x512, the per-tile
-// kernel's time first: 8-8-8-8-3 573 -> 259 us, 8-16-16-16-3 636 -> 354 us,
-// 8-32-32-32-3 790 -> 743 us; one 7-40-40-3 GELU image and one 256x256
-// 4-16-16-3 image are within 2 % of it.  Bound by issue, latency and the L1
-// data pipe: 306 warp instructions per 32 pixels of the 16-wide net at 0.57 a
-// cycle, and 78 % of the pipe's rate before the weights moved to registers.
+// kernel's time first: 8-8-8-8-3 573 -> 283 us, 8-16-16-16-3 636 -> 403 us,
+// 8-32-32-32-3 790 -> 771 us; one 7-40-40-3 GELU image with L2 flushed 37.5 ->
+// 31.4 us, one 256x256 4-16-16-3 image 10.9 -> 8.8 us.  Bound by issue, latency
+// and the L1 data pipe (74 % of its rate): 364 warp instructions per 32 pixels
+// of the 16-wide net at 0.60 a cycle.
 //
 // Precision is that of the per-tile tcgen05 kernels: fp16 weights as given, every
 // activation that an MMA reads as hi + lo fp16 terms (~22 bits, values below

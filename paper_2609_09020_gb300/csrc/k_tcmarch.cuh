@@ -30,15 +30,15 @@
 //
 // What bounds it: the chain of a tile's two (or more) remaining round trips
 // with four tiles in flight -- tensor memory holds no more -- and, next to
-// it, the splits.  A 7-64-64-3 tile takes about 980 cycles a group slot:
-// uncontended, its chain is 200 (wait for layer 0) + 410 (epilogue) + 745
-// (hidden layer, nine MMAs) + 340 + 395 (output layer) + 265 cycles, four
-// of which share one tensor pipe (about 540 cycles a tile in such small
-// batches) and the issue slots (680 warp instructions a tile and warp, 0.68
-// a cycle).  64 images of 768x512: 705 us with the per-tile kernel, whose
-// decoding warps also staged and interpolated the features, 660 us here;
-// 14-64-64-3 at 1361x2041, two images: 228 -> 174 us; 16-64-64-64-3 GELU at
-// 3840x2160, bound by the GELUs: 1020 -> 990 us (789 with the GELU of
+// it, the splits.  An SM finishes a 7-64-64-3 tile every 1,070 cycles.
+// Uncontended, a tile's chain is 200 (wait for layer 0) + 410 (epilogue) + 745
+// (hidden layer, nine MMAs) + 340 + 395 (output layer) + 265 cycles; four
+// of them share one tensor pipe (about 540 cycles a tile in such small
+// batches) and the issue slots (720 warp instructions per 32 pixels, 0.73
+// a cycle).  64 images of 768x512: 701 us with the per-tile kernel, whose
+// decoding warps also staged and interpolated the features, 668 us here;
+// 14-64-64-3 at 1361x2041, two images: 228 -> 175 us; 16-64-64-64-3 GELU at
+// 3840x2160, bound by the GELUs: 1021 -> 789 us (990 without the GELU of
 // pic_common.cuh and the operands in two parts).
 // Both thin layers, or the output layer alone, by warp-level mma.sync on
 // accumulator fragments (one round trip less) measured 740 and 779 us:
@@ -77,8 +77,9 @@ struct MarchNet {
   // ahead of the rest: the MMAs of the first part, and the better part of
   // their round trip, run beside the rest of the epilogue.  16-64-64-64-3 GELU
   // at 3840x2160: 836 us in one part, 789 cut after 16 columns, 825 after 32,
-  // 890 after 48; 7-64-64-3, one 768x512 image 20.4 -> 19.1 us, 64 of them
-  // the same; 14-64-64-3, one image of 1361x2041 70.0 -> 67.5 us.
+  // 890 after 48; 7-64-64-3, one 768x512 image 20.4 -> 18.8 us, 64 of them
+  // the same; 14-64-64-3, one image of 1361x2041 70.0 -> 66.7 us (all before
+  // layer 0 waited for the last layer).
   static constexpr int CUT = 1;
   static constexpr int THREADS = 32 * (kDecWarps + kFeatWarps + kGroups);
   // 896 threads x 72 registers at launch, moved between the roles'
